@@ -797,81 +797,56 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         if (!wait_group(G + j, 8)) goto softmax_done;
         tc_fence_after();
         const uint32_t t_s = tmem + lane_off + kColS + static_cast<uint32_t>(kBN) * b;
-        // this thread's columns of S in s[]; with two halves, the other half's
-        // maximum in m_other
+        // this thread's columns of S in s[] and the row's maximum in m_raw.  The
+        // loads deliver the maximum of each 32 columns (tcgen05.ld.red), which
+        // only a tile with keys past the end of its range cannot use.  The
+        // maximum sits on the latency loop that bounds the kernel (S ready ->
+        // softmax -> P -> next S): with 96 max instructions per 192-key tile it
+        // took about 190 of 2142 cycles.  Step at 4608 live and 20480 cached
+        // rows, 24 heads: 898 -> 838 us (E4M3 cache, where each half of a row
+        // finds the maximum of the whole row: 1040 -> 995 us), same bits.
         float s[kC];
-        float m_other = -INFINITY;
-        if constexpr (kH == 1) {
-          uint32_t r[kC / 32][32];
+        float m_raw;
+        auto chunk_max = [&](const float* x) -> float {
+          float m = fmax3(x[0], x[1], x[2]);
 #pragma unroll
-          for (int k = 0; k < kC / 32; ++k) tmem_ld32(t_s + 32u * k, r[k]);
+          for (int c = 3; c < 31; c += 2) m = fmax3(m, x[c], x[c + 1]);
+          return fmaxf(m, x[31]);
+        };
+        {
+          // with two halves, also the other half's columns, for the maximum only
+          constexpr int kChains = kBN / 32;
+          uint32_t r[kChains][32];
+          float mx[kChains];
 #pragma unroll
-          for (int k = 0; k < kC / 32; ++k) tmem_wait_ld(r[k]);
+          for (int k = 0; k < kChains; ++k) {
+            const uint32_t col = static_cast<uint32_t>(kH == 1 ? 32 * k : (col0 + 32 * k) & (kBN - 1));
+            tmem_ld32_max(t_s + col, r[k], mx[k]);
+          }
+#pragma unroll
+          for (int k = 0; k < kChains; ++k) tmem_wait_ld(r[k], mx[k]);
 #pragma unroll
           for (int k = 0; k < kC / 32; ++k)
 #pragma unroll
             for (int c = 0; c < 32; ++c) s[32 * k + c] = __uint_as_float(r[k][c]);
           if (src.valid < kBN) {  // keys past the end of the range
 #pragma unroll
-            for (int c = 0; c < kC; ++c)
-              if (c >= src.valid) s[c] = -INFINITY;
-          }
-        } else {
-          // own 64 columns, and the other half's 64 for the maximum only
-          const uint32_t other = static_cast<uint32_t>(kC - col0);
-          uint32_t r0[32], r1[32], x0[32], x1[32];
-          tmem_ld32(t_s + static_cast<uint32_t>(col0), r0);
-          tmem_ld32(t_s + static_cast<uint32_t>(col0) + 32u, r1);
-          tmem_ld32(t_s + other, x0);
-          tmem_ld32(t_s + other + 32u, x1);
-          tmem_wait_ld(r0);
-          tmem_wait_ld(r1);
-          tmem_wait_ld(x0);
-          tmem_wait_ld(x1);
-          float o[64];
+            for (int k = 0; k < kChains; ++k) {
+              float x[32];
+              const int col = kH == 1 ? 32 * k : (col0 + 32 * k) & (kBN - 1);
 #pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            s[c] = __uint_as_float(r0[c]);
-            s[32 + c] = __uint_as_float(r1[c]);
-            o[c] = __uint_as_float(x0[c]);
-            o[32 + c] = __uint_as_float(x1[c]);
-          }
-          if (src.valid < 128) {  // keys past the end of the range
-#pragma unroll
-            for (int c = 0; c < 64; ++c) {
-              if (col0 + c >= src.valid) s[c] = -INFINITY;
-              if (static_cast<int>(other) + c >= src.valid) o[c] = -INFINITY;
+              for (int c = 0; c < 32; ++c) {
+                x[c] = col + c < src.valid ? __uint_as_float(r[k][c]) : -INFINITY;
+                if (k < kC / 32) s[32 * k + c] = x[c];
+              }
+              mx[k] = chunk_max(x);
             }
           }
-          float mx[2];
-#pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            mx[k] = fmax3(o[32 * k], o[32 * k + 1], o[32 * k + 2]);
-#pragma unroll
-            for (int c = 3; c < 31; c += 2) mx[k] = fmax3(mx[k], o[32 * k + c], o[32 * k + c + 1]);
-            mx[k] = fmaxf(mx[k], o[32 * k + 31]);
-          }
-          m_other = fmaxf(mx[0], mx[1]);
-        }
-        // the row maximum of the raw scores: four independent chains of
-        // 3-input max over this thread's columns (and the other half's maximum)
-        auto row_max = [&]() -> float {
-          constexpr int kChains = kC / 32;
-          float mx[kChains];
-#pragma unroll
-          for (int k = 0; k < kChains; ++k) {
-            mx[k] = fmax3(s[32 * k], s[32 * k + 1], s[32 * k + 2]);
-#pragma unroll
-            for (int c = 3; c < 31; c += 2) mx[k] = fmax3(mx[k], s[32 * k + c], s[32 * k + c + 1]);
-            mx[k] = fmaxf(mx[k], s[32 * k + 31]);
-          }
           if constexpr (kChains == 6)
-            return fmax3(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[5]), -INFINITY);
-          else if constexpr (kChains == 4)
-            return fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
+            m_raw = fmaxf(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[5]));
           else
-            return fmax3(mx[0], mx[1], m_other);
-        };
+            m_raw = fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
+        }
         // rescale this row's O columns and l for a new running maximum m_new (O
         // must first hold P_j-1 V_j-1: group G + j + 1 complete)
         auto rescale = [&](float m_new) -> bool {
@@ -951,7 +926,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         };
         // running maximum from the row maximum (lazy: moves only when a tile's
         // maximum exceeds it by more than 2^8)
-        const float m_tile = fmaf(row_max(), c_t, shift);
+        const float m_tile = fmaf(m_raw, c_t, shift);
         if (j == 0) {
           m_run = m_tile;
         } else if (__any_sync(0xffffffffu, m_tile > m_run + 8.0f)) {

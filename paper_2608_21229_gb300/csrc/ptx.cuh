@@ -93,11 +93,28 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
       : "r"(taddr)
       : "memory");
 }
+// The same, with the maximum (as fp32) of the 32 columns found on the way
+// (tcgen05.ld.red).
+__device__ __forceinline__ void tmem_ld32_max(uint32_t taddr, uint32_t (&r)[32], float& mx) {
+  asm volatile(
+      "tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, %32, [%33];"
+      : RC_R8(0), RC_R8(8), RC_R8(16), RC_R8(24), "=f"(mx)
+      : "r"(taddr)
+      : "memory");
+}
 // Wait for this thread's outstanding TMEM loads; the registers are threaded
 // through so that no use of them can be scheduled before the wait.
 __device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : RC_P8(0), RC_P8(8), RC_P8(16), RC_P8(24)
+               :
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[32], float& mx) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : RC_P8(0), RC_P8(8), RC_P8(16), RC_P8(24), "+f"(mx)
                :
                : "memory");
 }

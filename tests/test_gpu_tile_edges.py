@@ -1,0 +1,57 @@
+"""Key ranges that end inside a key tile, with far higher scores just past the
+end: the tile holds rows of the next request there, and none of them may enter
+the row maximum (which the kernels take from the loads of whole 32-column
+chunks).  A maximum that included one would exceed the row's own by more than
+2^100 and every visible weight would vanish.  Bars as in the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import workloads
+from paper_2608_21229_gb300 import refcache as rcb
+
+import parity_utils as pu
+import test_gpu_fp8 as fp8
+
+pytestmark = pytest.mark.gpu
+
+#: (live keys, reference keys) of the first request: below, at and above the
+#: edges of 32-column chunks and of 128- and 192-key tiles
+LENGTHS = [(1, 193), (31, 192), (32, 191), (33, 129), (96, 97), (127, 128), (128, 127), (129, 33), (191, 32), (192, 31), (193, 1)]
+GAIN = 30.0  # the second request's keys: its scores have 30 times the first's spread
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.fail("GPU tests need a CUDA device")
+    rcb.load()
+    oracle.build()
+    yield
+    rcb.set_kernel("tcgen05")
+
+
+def _workload(n_x, n_r, head_dim):
+    w = workloads.Workload(f"edges_{n_x}_{n_r}", 2, head_dim,
+                           (workloads.Request(0, 0, n_x, n_r), workloads.Request(0, 0, 200, 200)), 31)
+    static, live = list(workloads.static_qkv(w)), list(workloads.live_qkv(w))
+    for t, first in ((static[1], n_r), (live[1], n_x)):
+        t[first:] = (t[first:].float() * GAIN).to(torch.bfloat16)
+    return w, tuple(static), tuple(live)
+
+
+@pytest.mark.parametrize("kernel", ["tcgen05", "tcgen05_k128"])
+@pytest.mark.parametrize("head_dim", [64, 128])
+@pytest.mark.parametrize("lengths", LENGTHS, ids=str)
+def test_keys_past_the_end_do_not_enter_the_maximum(kernel, head_dim, lengths):
+    w, static, live = _workload(*lengths, head_dim)
+    pu.full_compare(pu.GpuRun(w, kernel=kernel, static=static, live=live))
+
+
+@pytest.mark.parametrize("lengths", LENGTHS, ids=str)
+def test_keys_past_the_end_do_not_enter_the_maximum_e4m3(monkeypatch, lengths):
+    w, static, live = _workload(*lengths, 128)
+    rcb.set_kernel("tcgen05")
+    monkeypatch.setattr(workloads, "live_qkv", lambda *a, **k: live)
+    fp8.check_step(fp8.Fp8Run(w, static=static), np.arange(2), statistical=False)
