@@ -75,8 +75,21 @@
 //                      has finished reading O for the previous item, and (the
 //                      leader's warp 0 waited for it) the stage of P_t V_t's
 //                      group is full.
+//   p_half[t % 2]      192-key tiles: the same for P's first 32 keys, whose
+//                      P.V MMAs are issued while the softmax works on the rest
 //   stage_full[s]      the producers' TMA bytes of both CTAs (leader's barrier)
 //   q_full / q_empty   per Q buffer, once per item
+//
+// P in two pieces (192-key tiles): a tile's P.V and the S that reuses its
+// buffer (1536 tensor cycles) cannot start before its softmax is done, and with
+// two S buffers that loop -- S ready, softmax, P, MMAs, next S ready -- set the
+// period: 1880 cycles per tile at 4608 live and 20480 cached rows, 24 heads, of
+// which the MMA thread waited 480 for P.  With the first 32 keys handed over
+// early, their handshake, the stage check and the start of the P.V MMAs leave
+// the loop: 1698 cycles per tile, 143 of them waiting.  Larger first pieces are
+// no faster (64 keys 1693, 96 keys 1710, 128 keys 1757 cycles) and slower in
+// time where power sets the clock (interleaved, one run: 32 keys 875 us, 64
+// keys 924, 96 keys 914, one piece 956).
 //
 // E4M3 cache (kF8): key range B is the quantised reference cache -- K as
 // E4M3 codes [rows_pad, H, 128] and V transposed per head [H, 128, rows_pad],
@@ -136,6 +149,9 @@ struct Cfg {
   static constexpr uint32_t kColP = kPOverS ? 0u : 256u; // P buffer b at kColP + b * kPStride
   static constexpr uint32_t kPStride = kPOverS ? kBN : 64u;
   static constexpr uint32_t kColO = 384;
+  // 32-key chunks of P handed over ahead of the rest (0: P in one piece), see
+  // the head of the file
+  static constexpr int kPSplit = kPOverS ? 1 : 0;
   static_assert(2 * kBN <= 384 && kColO + kD <= tc::kTmemCols, "tensor-memory layout");
 };
 constexpr int kPairDoneBars = 4;          // pair_done[g % 4]: a waiter for group g holds up group g + 4
@@ -157,7 +173,7 @@ struct SmemT {
   static constexpr uint32_t kLX = kScales + (kF8 ? kScaleSlots * 16u : 0u);  // [2][128] fp32 partial row sums
   static constexpr uint32_t kBars = kLX + (kF8 ? 2u * 128u * 4u : 0u);
   static constexpr int kQFull = 0, kQEmpty = 2, kStageFull = 4, kPairDone = 4 + kStages,
-                       kPFull = kPairDone + kPairDoneBars, kMmaDone = kPFull + 2, kQ8Full = kMmaDone + 1,
+                       kPFull = kPairDone + kPairDoneBars, kPHalf = kPFull + 2, kMmaDone = kPHalf + 2, kQ8Full = kMmaDone + 1,
                        kLXFull = kQ8Full + 1, kScaleFull = kLXFull + 1, kScaleEmpty = kScaleFull + kScaleSlots,
                        kItemFull = kScaleEmpty + kScaleSlots, kItemEmpty = kItemFull + kItemSlots,
                        kNumBars = kItemEmpty + kItemSlots;
@@ -263,6 +279,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   constexpr int kStages = Cfg::kStages;
   constexpr uint32_t kColS = Cfg::kColS, kColP = Cfg::kColP, kPStride = Cfg::kPStride, kColO = Cfg::kColO;
   constexpr int kWarpArrivals = Cfg::kWarpArrivals;
+  constexpr int kPSplit = Cfg::kPSplit;
   using tc2::group_parity;
   using tc2::wait_cl;
   using tc2::wait_cl_warp;
@@ -305,6 +322,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       mbar_init(bar(L::kQFull + i), 1);
       mbar_init(bar(L::kQEmpty + i), 1);
       mbar_init(bar(L::kPFull + i), kWarpArrivals);
+      mbar_init(bar(L::kPHalf + i), kWarpArrivals);
     }
     for (int s = 0; s < kStages; ++s) mbar_init(bar(L::kStageFull + s), 1);
     for (int s = 0; s < tc2::kPairDoneBars; ++s) mbar_init(bar(L::kPairDone + s), 1);
@@ -564,14 +582,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         // also covers this group's stage and the previous item's O reads)
         for (int j = 0; j < nkv; ++j, ++g) {
           if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
+          const int t = t0 + j;
+          const int slot = stage_of(g);
+          const uint64_t soff = static_cast<uint64_t>(slot) * (kStage >> 4);
+          const uint64_t vd = vd0 + soff;
+          const uint32_t a_p = tmem + kColP + static_cast<uint32_t>(t & 1) * kPStride;
+          const uint32_t acc0 = j > 0 ? 1u : 0u;
+          if constexpr (kPSplit > 0) {  // P's first chunks
+            if (lane == 0) {
+              tc_fence_after();
+#pragma unroll
+              for (int kk = 0; kk < 2 * kPSplit; ++kk)
+                tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+            }
+            issued = true;
+            __syncwarp();
+            if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
+          }
           if (lane == 0) {
-            const int t = t0 + j;
             tc_fence_after();
-            const int slot = stage_of(g);
-            const uint64_t soff = static_cast<uint64_t>(slot) * (kStage >> 4);
-            const uint64_t vd = vd0 + soff;
-            const uint32_t a_p = tmem + kColP + static_cast<uint32_t>(t & 1) * kPStride;
-            const uint32_t acc0 = j > 0 ? 1u : 0u;
             const bool pv8 = kF8 && j >= na;      // P_j V_j on E4M3 operands
             const bool s8 = kF8 && j + 2 >= na;   // S_j+2 on E4M3 operands
             const uint64_t vd8 = vd80 + soff;
@@ -581,7 +610,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
               if (!s8 && Cfg::kPOverS) {
                 // S_j+2 overwrites P_j: every P.V MMA of the group goes first
 #pragma unroll
-                for (int kk = 0; kk < kBN / 16; ++kk)
+                for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
                   tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
 #pragma unroll
                 for (int kk = 0; kk < DG / 16; ++kk)
@@ -613,7 +642,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                 tc2_mma_ts_f8(tmem + kColO, a_p + 8u * kk, vd8 + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : acc0);
             } else {
 #pragma unroll
-              for (int kk = 0; kk < kBN / 16; ++kk)
+              for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
                 tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
             }
             tc2_commit_mc(bar(L::kPairDone + (g & 3)), 3);
@@ -661,6 +690,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         }
         for (int j = 0; j < nkv; ++j, ++g) {
           const int t = t0 + j;
+          if constexpr (kPSplit > 0) {
+            ok = wait_cl_warp(bar(L::kStageFull + stage_of(g)), stage_parity(g), ctl, 13);
+            ok = ok && wait_cl_warp(bar(L::kPHalf + (t & 1)), static_cast<uint32_t>(t >> 1) & 1u, ctl, 22);
+            if (bar_red_or(tc2::kGateBarrier, 64, !ok)) goto gate_done;
+          }
           ok = wait_cl_warp(bar(L::kPFull + (t & 1)), static_cast<uint32_t>(t >> 1) & 1u, ctl, 7);
           if (q8 && j + 2 == na) ok = ok && wait_cl_warp(bar(L::kQ8Full), q8_parity, ctl, 14);
           if (bar_red_or(tc2::kGateBarrier, 64, !ok)) goto gate_done;
@@ -878,6 +912,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         // columns at a time), or for a cached tile E4M3 quads (32 keys = 8
         // columns); returns this thread's sum of the weights written
         const uint32_t t_p = tmem + lane_off + kColP + kPStride * b;
+        auto p_arrive = [&](int which) {  // this warp's P so far is in TMEM
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(mapa_shared(bar(which), 0));
+        };
         auto write_p = [&]() -> float {
           const float bias = (kF8 ? shift + wshift : 0.f) - m_run;
           const f32x2 negm = make_f32x2(bias, bias);
@@ -917,6 +957,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                 pk[c] = pack_bf16x2(x, y);
               }
               tmem_st16(t_p + static_cast<uint32_t>(col0 / 2) + 16u * k, pk);
+              if (k == kPSplit - 1) p_arrive(L::kPHalf + b);
             }
           }
           const f32x2 l2 = add_f32x2(add_f32x2(lacc[0], lacc[1]), add_f32x2(lacc[2], lacc[3]));
@@ -936,13 +977,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         l_run += kF8 ? l_tile * lscale : l_tile;
         // the MMA thread waits only for P: the leader's warp 0 first makes
         // sure that the stage of P_j V_j's group (G + j + 2) has landed
-        if (leader && warp == 0 &&
+        if (kPSplit == 0 && leader && warp == 0 &&
             !wait_warp(bar(L::kStageFull + stage_of(G + j + 2)), stage_parity(G + j + 2), ctl, 13))
           goto softmax_done;
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(mapa_shared(bar(L::kPFull + b), 0));
+        p_arrive(L::kPFull + b);
       }
       {
         // the row's place: the bf16 kernels read it again from the work list, so
