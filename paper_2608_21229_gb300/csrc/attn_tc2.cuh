@@ -226,20 +226,9 @@ __device__ __forceinline__ int stage_of(int g) { return g % kStages; }
 template <int kStages>
 __device__ __forceinline__ uint32_t stage_parity(int g) { return static_cast<uint32_t>(g / kStages) & 1u; }
 
-// Bounded wait with cluster-scope acquire (barriers other CTAs arrive on).
+// Bounded wait on a barrier that other CTAs arrive on.
 __device__ __forceinline__ bool wait_cl(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  for (;;) {
-    for (int i = 0; i < 16; ++i)
-      if (mbar_try_wait_cluster(bar, parity)) return true;
-    if (*c.abort_flag) return false;
-    if (globaltimer_ns() - t0 > c.timeout_ns) {
-      *c.abort_flag = 1;
-      tc::report_timeout(c.status, where);
-      return false;
-    }
-  }
+  return tc::wait_one(bar, parity, c, where);
 }
 __device__ __forceinline__ bool wait_cl_warp(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
   const bool ok = wait_cl(bar, parity, c, where);
@@ -831,9 +820,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         if (!wait_group(G + j, 8)) goto softmax_done;
         tc_fence_after();
         const uint32_t t_s = tmem + lane_off + kColS + static_cast<uint32_t>(kBN) * b;
+        // Keys past the end of the range: -inf, written over their scores in
+        // tensor memory (a tile with such keys is rare; selects over the loaded
+        // columns were 8 KB of code inside the loop, see wait_more).
+        if (src.valid < kBN) {
+          uint32_t inf[16];
+#pragma unroll
+          for (int c = 0; c < 16; ++c) inf[c] = 0xFF800000u;
+          int c = src.valid;
+#pragma unroll 1
+          for (; c & 15; ++c) tmem_st1(t_s + static_cast<uint32_t>(c), 0xFF800000u);
+#pragma unroll 1
+          for (; c < kBN; c += 16) tmem_st16(t_s + static_cast<uint32_t>(c), inf);
+          tmem_wait_st();
+        }
         // this thread's columns of S in s[] and the row's maximum in m_raw.  The
-        // loads deliver the maximum of each 32 columns (tcgen05.ld.red), which
-        // only a tile with keys past the end of its range cannot use.  The
+        // loads deliver the maximum of each 32 columns (tcgen05.ld.red).  The
         // maximum sits on the latency loop that bounds the kernel (S ready ->
         // softmax -> P -> next S): with 96 max instructions per 192-key tile it
         // took about 190 of 2142 cycles.  Step at 4608 live and 20480 cached
@@ -841,12 +843,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         // finds the maximum of the whole row: 1040 -> 995 us), same bits.
         float s[kC];
         float m_raw;
-        auto chunk_max = [&](const float* x) -> float {
-          float m = fmax3(x[0], x[1], x[2]);
-#pragma unroll
-          for (int c = 3; c < 31; c += 2) m = fmax3(m, x[c], x[c + 1]);
-          return fmaxf(m, x[31]);
-        };
         {
           // with two halves, also the other half's columns, for the maximum only
           constexpr int kChains = kBN / 32;
@@ -863,19 +859,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           for (int k = 0; k < kC / 32; ++k)
 #pragma unroll
             for (int c = 0; c < 32; ++c) s[32 * k + c] = __uint_as_float(r[k][c]);
-          if (src.valid < kBN) {  // keys past the end of the range
-#pragma unroll
-            for (int k = 0; k < kChains; ++k) {
-              float x[32];
-              const int col = kH == 1 ? 32 * k : (col0 + 32 * k) & (kBN - 1);
-#pragma unroll
-              for (int c = 0; c < 32; ++c) {
-                x[c] = col + c < src.valid ? __uint_as_float(r[k][c]) : -INFINITY;
-                if (k < kC / 32) s[32 * k + c] = x[c];
-              }
-              mx[k] = chunk_max(x);
-            }
-          }
           if constexpr (kChains == 6)
             m_raw = fmaxf(fmax3(mx[0], mx[1], mx[2]), fmax3(mx[3], mx[4], mx[5]));
           else
