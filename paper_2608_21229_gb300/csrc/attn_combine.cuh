@@ -7,8 +7,12 @@
 // its keys.  Over all keys of the item the softmax normaliser is
 // l = sum_p exp(L_p), so the item's output is
 //   O = sum_p exp(L_p - L) O_p   with   L = log sum_p exp(L_p),
-// computed here with L_max subtracted first: one warp per query row, D / 32
-// head-dim columns per lane.
+// computed here with L_max subtracted first.
+//
+// Parts lie in the workspace as [part][D / 4][rows_per_part] float4 (the layout
+// in which the attention kernel's epilogue, a row per thread, writes whole
+// lines); a warp takes 32 rows and reads runs of 512 bytes, and the outputs go
+// through shared memory so that rows are written whole.
 #pragma once
 #include <cuda_bf16.h>
 
@@ -18,71 +22,75 @@
 namespace rc {
 
 constexpr int kMaxParts = 8;
+constexpr int kCombineRows = 32;
 
-// grid = (ceil(rows / 8), jobs), 256 threads: one warp per query row, all
-// parts' loads issued before any is used.
+// grid = (ceil(rows / 32), jobs), 256 threads: lane = row, warp w takes the
+// column quads w, w + 8, ...
 template <int D>
 __global__ void __launch_bounds__(256) combine_parts_kernel(const CombineJob* __restrict__ jobs,
                                                             const float* __restrict__ part_o,
                                                             const float* __restrict__ part_lse, int rows_per_part,
                                                             __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                                                             int64_t row_stride, int num_heads) {
-  static_assert(D == 128 || D == 64, "four or two columns per lane");
-  constexpr int kC = D / 32;
+  static_assert(D == 128 || D == 64, "four or two column quads per thread");
+  constexpr int kQ = D / 32;        // column quads of this thread
+  constexpr int kPitch = D + 8;     // bf16 elements of a staged row (16 bytes of padding)
+  __shared__ __align__(16) __nv_bfloat16 tile[kCombineRows * kPitch];
+  const CombineJob job = jobs[blockIdx.y];  // written when the cache was created
+  const int r0 = blockIdx.x * kCombineRows, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r = r0 + lane;
   grid_dependency_wait();  // the attention kernel's parts are complete
   if (threadIdx.x == 0) grid_launch_dependents();
-  const CombineJob job = jobs[blockIdx.y];
-  const int r = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (r >= job.q_rows) return;
+  if (r0 >= job.q_rows) return;
+  const bool ok = r < job.q_rows;
   const int np = min(job.nparts, kMaxParts);
-  float L[kMaxParts];
-  float v[kMaxParts][kC];
+  float w[kMaxParts];
+  float lmax = -INFINITY;
 #pragma unroll
   for (int p = 0; p < kMaxParts; ++p) {
-    if (p < np) {
-      const int64_t row = static_cast<int64_t>(job.part0 + p) * rows_per_part + r;
-      L[p] = part_lse[row];
-      if constexpr (kC == 4) {
-        const float4 x = reinterpret_cast<const float4*>(part_o + row * D)[lane];
-        v[p][0] = x.x, v[p][1] = x.y, v[p][2] = x.z, v[p][3] = x.w;
-      } else {
-        const float2 x = reinterpret_cast<const float2*>(part_o + row * D)[lane];
-        v[p][0] = x.x, v[p][1] = x.y;
-      }
-    } else {
-      L[p] = -INFINITY;
-#pragma unroll
-      for (int c = 0; c < kC; ++c) v[p][c] = 0.f;
-    }
+    w[p] = p < np && ok ? part_lse[static_cast<int64_t>(job.part0 + p) * rows_per_part + r] : -INFINITY;
+    lmax = fmaxf(lmax, w[p]);
   }
-  float lmax = L[0];
-#pragma unroll
-  for (int p = 1; p < kMaxParts; ++p) lmax = fmaxf(lmax, L[p]);
-  float acc[kC];
-#pragma unroll
-  for (int c = 0; c < kC; ++c) acc[c] = 0.f;
   float wsum = 0.f;
 #pragma unroll
   for (int p = 0; p < kMaxParts; ++p) {
-    const float w = p < np ? expf(L[p] - lmax) : 0.f;
-    wsum += w;
+    w[p] = p < np && ok ? expf(w[p] - lmax) : 0.f;
+    wsum += w[p];
+  }
+  float4 acc[kQ];
 #pragma unroll
-    for (int c = 0; c < kC; ++c) acc[c] += w * v[p][c];
+  for (int c = 0; c < kQ; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4* src = reinterpret_cast<const float4*>(part_o) +
+                      (static_cast<int64_t>(job.part0) * (D / 4) + warp) * rows_per_part + r;
+#pragma unroll
+  for (int p = 0; p < kMaxParts; ++p) {
+    if (p < np && ok) {
+#pragma unroll
+      for (int c = 0; c < kQ; ++c) {
+        const float4 x = src[(static_cast<int64_t>(p) * (D / 4) + 8 * c) * rows_per_part];
+        acc[c].x += w[p] * x.x, acc[c].y += w[p] * x.y, acc[c].z += w[p] * x.z, acc[c].w += w[p] * x.w;
+      }
+    }
   }
   const float inv = 1.0f / wsum;
-  const int64_t row = static_cast<int64_t>(job.q_row0) + r;
-  __nv_bfloat16* dst = out + row * row_stride + static_cast<int64_t>(job.head) * D;
-  __nv_bfloat162 lo = __floats2bfloat162_rn(acc[0] * inv, acc[1] * inv);
-  if constexpr (kC == 4) {
-    __nv_bfloat162 hi = __floats2bfloat162_rn(acc[2] * inv, acc[3] * inv);
+#pragma unroll
+  for (int c = 0; c < kQ; ++c) {
     uint2 packed;
-    packed.x = *reinterpret_cast<uint32_t*>(&lo);
-    packed.y = *reinterpret_cast<uint32_t*>(&hi);
-    reinterpret_cast<uint2*>(dst)[lane] = packed;
-  } else {
-    reinterpret_cast<__nv_bfloat162*>(dst)[lane] = lo;
+    packed.x = pack_bf16x2(acc[c].x * inv, acc[c].y * inv);
+    packed.y = pack_bf16x2(acc[c].z * inv, acc[c].w * inv);
+    *reinterpret_cast<uint2*>(&tile[lane * kPitch + 4 * (warp + 8 * c)]) = packed;
   }
-  if (lse && lane == 0) lse[row * num_heads + job.head] = lmax + logf(wsum);
+  if (lse && warp == 0 && ok)
+    lse[(static_cast<int64_t>(job.q_row0) + r) * num_heads + job.head] = lmax + logf(wsum);
+  __syncthreads();
+  constexpr int kNC = D / 8;  // 16-byte chunks of a row
+  for (int i = threadIdx.x; i < kCombineRows * kNC; i += 256) {
+    const int rr = i / kNC, ch = i % kNC;
+    if (r0 + rr < job.q_rows)
+      *reinterpret_cast<uint4*>(out + (static_cast<int64_t>(job.q_row0) + r0 + rr) * row_stride +
+                                static_cast<int64_t>(job.head) * D + 8 * ch) =
+          *reinterpret_cast<const uint4*>(&tile[rr * kPitch + 8 * ch]);
+  }
 }
 
 }  // namespace rc

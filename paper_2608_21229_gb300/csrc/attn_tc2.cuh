@@ -39,21 +39,31 @@
 // An item is a task of up to 256 query rows: CTA r takes rows
 // [128 r, 128 r + 128).  Items come from a per-item list ordered on the host
 // or, head-major, from the task list: with a work counter each CTA pair takes
-// the next item of the list whenever it starts one (the leader's producer
-// takes it and passes it on through a ring in shared memory), else pair c
-// takes items c, c + n_pairs, ...
+// its first item by its index and then the next of the list, else pair c takes
+// items c, c + n_pairs, ...  The leader's producer chooses them and passes each
+// item's Task on through a ring in both CTAs' shared memory.
 //
 // Work is done item by item (an item = a task of up to 256 rows x one
-// head).  An item with n key tiles is a sequence of n + 2 MMA groups:
-//   group G + 0, G + 1     S_0 = Q K_0^T, S_1 = Q K_1^T (the second is empty
-//                          when n = 1)
-//   group G + 2 + j        O += P_j V_j with S_j+2 = Q K_j+2^T when j + 2 < n
-//                          (all P.V MMAs first when S_j+2 overwrites P_j,
-//                          else interleaved MMA by MMA)
-// numbered g = 0, 1, 2, ... over all items of the cluster.  Group g reads
-// ring stage g % kStages (K of its S, V of its P.V; 48 KB per CTA at 192-key
-// tiles, 32 KB at 128).  Tiles are also numbered over all items (t); S_t and
-// P_t live in TMEM buffer t % 2.
+// head).  An item with n key tiles is a sequence of n + 1 MMA groups:
+//   group G               S_1 = Q K_1^T (empty when n = 1)
+//   group G + 1 + j       O += P_j V_j, then S_j+2 = Q K_j+2^T when j + 2 < n;
+//                         beside P_n-2 V_n-2 (or in group G when n = 1) the
+//                         next item's S_0
+// numbered g = 0, 1, 2, ... over all items of the cluster; group 0 is the first
+// item's S_0 alone.  Tiles are numbered t over all items: K_t and V_t lie in
+// slot t % kStages of a K and a V ring (24 KB each per CTA at 192-key tiles, 16
+// KB at 128), S_t and P_t in TMEM buffer t % 2.
+//
+// Between items: an item's Q and first K tiles are loaded, and its S_0 is
+// issued, while the item before it still runs, so that only the epilogue (O
+// read, normalised and stored) and the next item's first softmax lie between
+// the last P.V of one item and the first of the next.  For that the item is
+// chosen a few tiles ahead and its Task travels through shared memory: taking
+// the item, passing it to the other CTA and reading its Task from global memory
+// in every role one after the other took about 5000 cycles per item, and the
+// epilogue's uncoalesced stores 2000.  MMA-thread waits around an item's start
+// went from 5100 to 2700 cycles; step with 1280 live and 2048 cached rows
+// (items of 9 tiles), 24 heads: 62.7 -> 60.7 us.
 //
 // Synchronisation is built so that the MMA thread does as little as possible
 // between its MMAs: a tcgen05.mma blocks its thread until the tensor core
@@ -66,26 +76,31 @@
 // the same group sequence and leave together, so neither can be left waiting);
 // the MMA thread then issues the group and commits once:
 //   pair_done[g % 4]   one commit per group (multicast to both CTAs): its S
-//                      is in TMEM, its P.V is in O, its stage and the P
+//                      is in TMEM, its P.V is in O, the ring slots and the P
 //                      buffer it read are free.  Four barriers, so that no
 //                      waiter can miss a phase: a waiter for group g holds up
 //                      group g + 4.
 //   p_full[t % 2]      one arrival per softmax warp of both CTAs.  Its phase
-//                      for tile t means P_t is in TMEM, every softmax thread
-//                      has finished reading O for the previous item, and (the
-//                      leader's warp 0 waited for it) the stage of P_t V_t's
-//                      group is full.
+//                      for tile t means P_t is in TMEM and every softmax thread
+//                      has finished reading O for the previous item.
 //   p_half[t % 2]      192-key tiles: the same for P's first 32 keys, whose
 //                      P.V MMAs are issued while the softmax works on the rest
-//   stage_full[s]      the producers' TMA bytes of both CTAs (leader's barrier)
-//   q_full / q_empty   per Q buffer, once per item
+//   k_full[s] v_full[s]  the producers' TMA bytes of both CTAs (leader's barriers)
+//   q_full             per Q buffer, once per item
+//   q_empty            per Q buffer: the item's last S has read it, and the
+//                      epilogue no longer stages O in it
+//   item_full / item_empty  per slot of the item ring
+// The values that MMA operands are computed from (tensor-memory base, warp
+// index, key tiles) pass through a shuffle, which tells the compiler that they
+// are the same in all lanes: operands of tcgen05.mma live in uniform registers,
+// and moving each of them there cost the MMA thread 300 cycles per tile.
 //
 // P in two pieces (192-key tiles): a tile's P.V and the S that reuses its
 // buffer (1536 tensor cycles) cannot start before its softmax is done, and with
 // two S buffers that loop -- S ready, softmax, P, MMAs, next S ready -- set the
 // period: 1880 cycles per tile at 4608 live and 20480 cached rows, 24 heads, of
 // which the MMA thread waited 480 for P.  With the first 32 keys handed over
-// early, their handshake, the stage check and the start of the P.V MMAs leave
+// early, their handshake, the V slot's check and the start of the P.V MMAs leave
 // the loop: 1698 cycles per tile, 143 of them waiting.  Larger first pieces are
 // no faster (64 keys 1693, 96 keys 1710, 128 keys 1757 cycles) and slower in
 // time where power sets the clock (interleaved, one run: 32 keys 875 us, 64
@@ -136,10 +151,10 @@ struct Cfg {
   static constexpr int kProducerWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1, kGateWarp = kSoftmaxWarps + 2;
   static constexpr int kThreads = 32 * (kSoftmaxWarps + 3);
   static constexpr int kWarpArrivals = 2 * kSoftmaxWarps;  // p_full / q8_full: every softmax warp of both CTAs
-  // warps that take each item from the ring (work counter): the leader's
-  // gate and softmax warps, the follower's producer and softmax warps
+  // warps that read each item from the ring: the leader's gate and softmax
+  // warps, the follower's producer and softmax warps
   static constexpr int kItemTakers = 2 + 2 * kSoftmaxWarps;
-  static constexpr int kStages = kBN == 128 ? 4 : 3;     // ring stages (shared memory: 2 Q + stages <= 227 KB)
+  static constexpr int kStages = kBN == 128 ? 4 : 3;     // K and V ring slots (shared memory: 2 Q + slots <= 227 KB)
   static constexpr uint32_t kKBox = (kBN / 2) * 128;     // one K box: kBN / 2 rows x 128 bytes
   static constexpr uint32_t kKHalf = 2 * kKBox;          // this CTA's kBN / 2 keys x 128 d of a K tile
   static constexpr uint32_t kVHalf = kBN * 64 * 2;       // kBN keys x this CTA's 64 d of a V tile
@@ -160,19 +175,19 @@ constexpr uint32_t kKHalf8 = 64 * 128;   // 8 KB: this CTA's 64 keys x 128 d of 
 constexpr uint32_t kVHalf8 = 64 * 128;   // 8 KB: this CTA's 64 d x 128 keys of an E4M3 V^T tile
 constexpr uint32_t kQ8Tile = 128 * 128;  // this CTA's 128 query rows as E4M3
 constexpr int kScaleSlots = 8;           // ring of per-tile scales of cached tiles (E4M3 kernel)
-constexpr int kItemSlots = 4;            // ring of items taken from the work counter
+constexpr int kItemSlots = 8;            // ring of items
 
 template <bool kF8, int kBN>
 struct SmemT {
   using C = Cfg<kF8, kBN>;
   static constexpr int kStages = C::kStages;
   static constexpr uint32_t kQ = 0;                // Q buffers 0 and 1 (this CTA's 128 rows)
-  static constexpr uint32_t kRing = 2 * kQTile;    // stage s: [K half | V half]
+  static constexpr uint32_t kRing = 2 * kQTile;    // slot s: [K half | V half]
   static constexpr uint32_t kQ8 = kRing + kStages * C::kStage;  // E4M3 Q tile (kF8 only)
   static constexpr uint32_t kScales = kQ8 + (kF8 ? kQ8Tile : 0u);  // ring of kScaleSlots x 16 B (kF8 only)
   static constexpr uint32_t kLX = kScales + (kF8 ? kScaleSlots * 16u : 0u);  // [2][128] fp32 partial row sums
   static constexpr uint32_t kBars = kLX + (kF8 ? 2u * 128u * 4u : 0u);
-  static constexpr int kQFull = 0, kQEmpty = 2, kStageFull = 4, kPairDone = 4 + kStages,
+  static constexpr int kQFull = 0, kQEmpty = 2, kKFull = 4, kVFull = kKFull + kStages, kPairDone = kVFull + kStages,
                        kPFull = kPairDone + kPairDoneBars, kPHalf = kPFull + 2, kMmaDone = kPHalf + 2, kQ8Full = kMmaDone + 1,
                        kLXFull = kQ8Full + 1, kScaleFull = kLXFull + 1, kScaleEmpty = kScaleFull + kScaleSlots,
                        kItemFull = kScaleEmpty + kScaleSlots, kItemEmpty = kItemFull + kItemSlots,
@@ -180,16 +195,17 @@ struct SmemT {
   static constexpr uint32_t kTmemHolder = kBars + 8 * kNumBars;
   static constexpr uint32_t kAbort = kTmemHolder + 4;
   // load record of each CTA of the pair (leader's copy read at teardown):
-  // per CTA [loads per stage (kStages) | own bytes of the last load per stage
-  // (kStages) | the other CTA's bytes of that load (kStages) | loads per Q
-  // buffer (2)]
-  static constexpr uint32_t kRecWords = 3 * kStages + 2;
+  // per CTA [loads per slot of the K and V rings (kRings) | own bytes of the
+  // last load per slot (kRings) | the other CTA's bytes of that load (kRings)
+  // | loads per Q buffer (2)]
+  static constexpr int kRings = 2 * kStages;
+  static constexpr uint32_t kRecWords = 3 * kRings + 2;
   static constexpr uint32_t kLoadRec = kAbort + 4;
-  // ring of taken items (work counter): slot k % kItemSlots holds item k of
-  // this cluster (-1: none left); the gate warp passes the MMA warp its item
-  static constexpr uint32_t kItemRing = kLoadRec + 2 * kRecWords * 4;
-  static constexpr uint32_t kGateItem = kItemRing + 4 * kItemSlots;
-  static constexpr uint32_t kUsed = kGateItem + 4;
+  // ring of items: slot k % kItemSlots holds item k of this cluster (a Task;
+  // head -1: none left); the gate warp passes the MMA warp its item's tiles
+  static constexpr uint32_t kItemRing = (kLoadRec + 2 * kRecWords * 4 + 15u) & ~15u;
+  static constexpr uint32_t kGateItem = kItemRing + 32 * kItemSlots;  // two of [key tiles, of range A, first S ahead, -]
+  static constexpr uint32_t kUsed = kGateItem + 32;
   static constexpr uint32_t kMaxDynamic = 232448;
   static constexpr uint32_t kDynamic = kUsed + 1024 < kMaxDynamic ? kUsed + 1024 : kMaxDynamic;
   static_assert(kUsed <= kMaxDynamic, "shared-memory layout too large");
@@ -220,11 +236,11 @@ __device__ __forceinline__ int n_key_tiles(const Task& t, int& na) {
 
 // Phase parity of pair_done[g % 4] for group g.
 __device__ __forceinline__ uint32_t group_parity(int g) { return static_cast<uint32_t>(g >> 2) & 1u; }
-// Ring stage of group g and the phase parity of its stage_full barrier.
+// Ring slot of tile t and the phase parity of its barrier.
 template <int kStages>
-__device__ __forceinline__ int stage_of(int g) { return g % kStages; }
+__device__ __forceinline__ int slot_of(int t) { return t % kStages; }
 template <int kStages>
-__device__ __forceinline__ uint32_t stage_parity(int g) { return static_cast<uint32_t>(g / kStages) & 1u; }
+__device__ __forceinline__ uint32_t slot_parity(int t) { return static_cast<uint32_t>(t / kStages) & 1u; }
 
 // Bounded wait on a barrier that other CTAs arrive on.
 __device__ __forceinline__ bool wait_cl(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
@@ -279,8 +295,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   constexpr int DG = kDG;      // head dim of the tensors
   static_assert(DG == D || (DG == 64 && !kF8), "head dim 128, or 64 (bf16 cache) padded to 128");
   constexpr int kQBoxes = DG / 64;  // 64-column boxes of a Q or K row loaded
-  auto stage_of = [](int g) -> int { return tc2::stage_of<kStages>(g); };
-  auto stage_parity = [](int g) -> uint32_t { return tc2::stage_parity<kStages>(g); };
+  auto slot_of = [](int t) -> int { return tc2::slot_of<kStages>(t); };
+  auto slot_parity = [](int t) -> uint32_t { return tc2::slot_parity<kStages>(t); };
   constexpr uint32_t kIdescS = idesc_bf16_f32(256, kBN, false);
   constexpr uint32_t kIdescO = idesc_bf16_f32(256, D, true);
   constexpr uint32_t kIdesc8 = idesc_e4m3_f32(256, 128);  // S and O of cached tiles (N = 128 keys or d)
@@ -293,7 +309,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   volatile int* abort_flag = reinterpret_cast<volatile int*>(base_ptr + L::kAbort);
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(base_ptr + L::kTmemHolder);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0);
   const int lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
@@ -309,11 +325,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(L::kQFull + i), 1);
-      mbar_init(bar(L::kQEmpty + i), 1);
+      mbar_init(bar(L::kQEmpty + i), 1 + Cfg::kSoftmaxWarps);  // its last S, and O staged in it written
       mbar_init(bar(L::kPFull + i), kWarpArrivals);
       mbar_init(bar(L::kPHalf + i), kWarpArrivals);
     }
-    for (int s = 0; s < kStages; ++s) mbar_init(bar(L::kStageFull + s), 1);
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(bar(L::kKFull + s), 1);
+      mbar_init(bar(L::kVFull + s), 1);
+    }
     for (int s = 0; s < tc2::kPairDoneBars; ++s) mbar_init(bar(L::kPairDone + s), 1);
     mbar_init(bar(L::kMmaDone), 1);
     mbar_init(bar(L::kQ8Full), kWarpArrivals);
@@ -330,8 +349,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     fence_barrier_init();
     fence_proxy_async_smem();
   }
+  if (warp == Cfg::kProducerWarp && lane == 0) {
+    prefetch_tmap(&tm_q);
+    prefetch_tmap(&tm_ka);
+    prefetch_tmap(&tm_va);
+    prefetch_tmap(&tm_kb);
+    prefetch_tmap(&tm_vb);
+  }
   if constexpr (DG != D) {
-    // head dim 64: the second CTA's V half of every stage is the zero padding
+    // head dim 64: the second CTA's V half of every ring slot is the zero padding
     // of the upper 64 head-dim columns (written once; that CTA never loads V)
     if (rank == 1) {
       constexpr uint32_t kChunks = kVHalf / 16;
@@ -353,59 +379,50 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   // is complete; and the next kernel may start its CTAs (they wait likewise)
   grid_dependency_wait();
   if (threadIdx.x == 0) grid_launch_dependents();
-  const uint32_t tmem = *tmem_holder;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);
   const Ctl ctl{abort_flag, args.timeout_ns, args.status};
   auto lbar = [&](int i) -> uint32_t { return mapa_shared(bar(i), 0); };  // leader's barrier i
-  // Item k of this cluster (k = 0, 1, ...; -1 once there is none, -2 after a
-  // failed wait).  Static order: cluster + k * n_clusters.  With a work
-  // counter the leader's producer takes the next item of the list for each k
-  // (atomic increment) and writes it to ring slot k % kItemSlots of both CTAs;
-  // the other warps read it there.  A slot is reused once every taker has
-  // read it (item_empty, on the leader).
+  // Items reach the warps that walk them through a ring in the shared memory
+  // of both CTAs: the leader's producer chooses item k, reads its Task and
+  // writes it to slot k % kItemSlots of both, well before the item is needed.
+  // Static order: item cluster + k * n_clusters.  With a work counter: item
+  // `cluster` first, then the next of the list (atomic increment).  A slot is
+  // reused once every taker is done with it (item_empty, on the leader).
   const bool dyn = args.work != nullptr;
-  volatile int* item_ring = reinterpret_cast<volatile int*>(base_ptr + L::kItemRing);
-  auto static_item = [&](int k) -> int {
-    const int64_t it = static_cast<int64_t>(cluster) + static_cast<int64_t>(k) * n_clusters;
-    return it < args.n_items ? static_cast<int>(it) : -1;
+  auto ring_slot = [&](int k) -> uint32_t {
+    return base + L::kItemRing + 32u * static_cast<uint32_t>(k % tc2::kItemSlots);
   };
-  auto publish_item = [&](int k) -> int {  // leader's producer (one thread)
-    const int s = k % tc2::kItemSlots;
-    if (k >= tc2::kItemSlots &&
-        !wait_cl(bar(L::kItemEmpty + s), static_cast<uint32_t>(k / tc2::kItemSlots - 1) & 1u, ctl, 21))
-      return -2;
-    int it = atomicAdd(args.work, 1);
-    if (it >= args.n_items) it = -1;
-    item_ring[s] = it;
-    st_cluster_u32(mapa_shared(base + L::kItemRing + 4u * static_cast<uint32_t>(s), 1), static_cast<uint32_t>(it));
-    mbar_arrive(bar(L::kItemFull + s));
-    mbar_arrive_release_cluster(mapa_shared(bar(L::kItemFull + s), 1));
-    return it;
+  auto ring_read = [&](int k) -> Task {
+    const uint4 lo = ld_shared_v4(ring_slot(k)), hi = ld_shared_v4(ring_slot(k) + 16u);
+    Task t;
+    t.q_row0 = static_cast<int>(lo.x), t.q_rows = static_cast<int>(lo.y);
+    t.a_row0 = static_cast<int>(lo.z), t.a_len = static_cast<int>(lo.w);
+    t.b_row0 = static_cast<int>(hi.x), t.b_len = static_cast<int>(hi.y);
+    t.head = static_cast<int>(hi.z), t.part = static_cast<int>(hi.w);
+    return t;
   };
-  auto take_item = [&](int k, int where) -> int {  // one thread of a taking warp
-    const int s = k % tc2::kItemSlots;
-    if (!wait_cl(bar(L::kItemFull + s), static_cast<uint32_t>(k / tc2::kItemSlots) & 1u, ctl, where)) return -2;
-    const int it = item_ring[s];
-    mbar_arrive_release_cluster(lbar(L::kItemEmpty + s));
-    return it;
+  // wait until item k is in the ring / this warp (one lane) is done with it
+  auto ring_wait = [&](int k, int where) -> bool {
+    const uint32_t full = bar(L::kItemFull + k % tc2::kItemSlots), parity = static_cast<uint32_t>(k / tc2::kItemSlots) & 1u;
+    // (complete after wait_cl; once more for the acquire of the leader's writes)
+    return wait_cl(full, parity, ctl, where) && (leader || mbar_try_wait_acquire_cluster(full, parity));
   };
-  auto take_item_warp = [&](int k, int where) -> int {
-    int it = 0;
-    if (lane == 0) it = dyn ? take_item(k, where) : static_item(k);
-    return __shfl_sync(0xffffffffu, it, 0);
-  };
+  auto ring_done = [&](int k) { mbar_arrive_cluster(lbar(L::kItemEmpty + k % tc2::kItemSlots)); };
 
   if (warp == Cfg::kProducerWarp) {
     // ------------------------------------------------------------ producer (both CTAs)
-    // This CTA's halves of the stages of every group, in group order, and an
-    // item's Q rows just before its first stage.
+    // This CTA's halves of the K and V tiles, and an item's Q rows just before
+    // its first K tile.  Tiles are numbered t over all items; step t loads V_t
+    // and K_t+2, which may belong to the next item, so that an item's first
+    // loads are in flight before the item before it ends.
     if (lane == 0) {
-      // loads this CTA issued per stage and per Q buffer, and its bytes of the
-      // last load of each stage; the leader arms every phase for both CTAs'
-      // bytes right before it issues its own half
-      int n_stage[kStages];
-      uint32_t own_bytes[kStages], other_bytes[kStages];
-      for (int s = 0; s < kStages; ++s) {
-        n_stage[s] = 0;
+      // loads this CTA issued per K slot, V slot and Q buffer, and both CTAs'
+      // bytes of the last load of each slot; the leader arms every phase for
+      // both CTAs' bytes right before it issues its own half
+      int n_ring[L::kRings];
+      uint32_t own_bytes[L::kRings], other_bytes[L::kRings];
+      for (int s = 0; s < L::kRings; ++s) {
+        n_ring[s] = 0;
         own_bytes[s] = 0;
         other_bytes[s] = 0;
       }
@@ -413,108 +430,180 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       int scale_armed[tc2::kScaleSlots];
       for (int s = 0; s < tc2::kScaleSlots; ++s) scale_armed[s] = -1;
       bool skip_next = leader && args.dbg_skip_first_load != 0;
-      int g = 0, qi = 0, si = 0;  // si: cached tiles whose scales went into the ring
-      Task tk;
-      int head = 0, na = 0;
-      // stage of group g: K tile kj (if kj >= 0) and V tile vj (if vj >= 0) of the item
-      auto load_stage = [&](int kj, int vj) -> bool {
-        const int slot = stage_of(g);
-        // the stage's previous group (g - kStages) must be complete
-        if (g >= kStages &&
-            !wait_one(bar(L::kPairDone + ((g - kStages) & 3)), group_parity(g - kStages), ctl, 2))
-          return false;
-        const uint32_t dst = base + L::kRing + static_cast<uint32_t>(slot) * kStage;
-        const uint32_t full = lbar(L::kStageFull + slot);
-        const TileSrc ks = tc2::tile_src<kBN>(tk, na, kj >= 0 ? kj : 0);
-        const TileSrc vs = tc2::tile_src<kBN>(tk, na, vj >= 0 ? vj : 0);
-        const bool k8 = kF8 && kj >= 0 && ks.in_b, v8 = kF8 && vj >= 0 && vs.in_b;
-        // each CTA's K bytes; a V half (at head dim 64 only the first CTA loads one)
-        const uint32_t kb = kj >= 0 ? (k8 ? kKHalf8 : kKBox * kQBoxes) : 0u;
-        const uint32_t vb = vj >= 0 ? (v8 ? kVHalf8 : kVHalf) : 0u;
-        const bool v_here = DG == D || rank == 0;
-        const uint32_t bytes = 2 * kb + (DG == D ? 2 : 1) * vb;  // both CTAs
-        if (k8) {
-          // this CTA's softmax warps read the cached tile's scales from ring slot
-          // si % kScaleSlots; the slot's previous tile must have been read
-          const int sl = si % tc2::kScaleSlots, use = si / tc2::kScaleSlots;
-          if (use > 0 && !wait_one(bar(L::kScaleEmpty + sl), static_cast<uint32_t>(use - 1) & 1u, ctl, 16)) return false;
-          mbar_arrive_expect_tx(bar(L::kScaleFull + sl), 16u);
-          scale_armed[sl] = use & 1;
-          bulk_load(base + L::kScales + 16u * static_cast<uint32_t>(sl),
-                    args.b_scales + ((tk.b_row0 >> 7) + (kj - na)) * args.num_heads + head, 16u,
-                    bar(L::kScaleFull + sl));
-          ++si;
-        }
-        if (skip_next) {  // fault injection: the leader never arms or loads this stage
-          skip_next = false;
+      int si = 0;  // cached tiles whose scales went into the ring
+      // The leader's choice of the next item, in three steps, each of whose
+      // result is first used by the following one: its index, its Task, its
+      // publication.
+      int n_pub = 0, pub_step = 0, pub_item = 0, pub_head = 0, pub_q = 0;
+      bool pub_end = false;
+      Task pub_task{};
+      auto pub_advance = [&]() -> bool {
+        if (pub_step == 0) {
+          const int64_t it = !dyn ? static_cast<int64_t>(cluster) + static_cast<int64_t>(n_pub) * n_clusters
+                             : n_pub == 0 ? static_cast<int64_t>(cluster)
+                                          : static_cast<int64_t>(n_clusters) + atomicAdd(args.work, 1);
+          pub_item = static_cast<int>(min(it, static_cast<int64_t>(args.n_items)));
+        } else if (pub_step == 1) {
+          if (pub_item < args.n_items)
+            decode_item(args, pub_item, pub_task, pub_head);
+          else
+            pub_head = -1;
         } else {
-          if (leader) mbar_arrive_expect_tx(bar(L::kStageFull + slot), bytes);
-          ++n_stage[slot];
-          own_bytes[slot] = kb + (v_here ? vb : 0u);
-          other_bytes[slot] = kb + (DG == D || rank == 1 ? vb : 0u);
-          if (k8) {  // E4M3 keys [64 r, 64 r + 64): one box of 64 rows x 128 bytes
-            tma_load_2d_pair(dst, &tm_kb, full, head * D, ks.row + 64 * static_cast<int>(rank));
-          } else if (kj >= 0) {  // keys [kBN/2 r, kBN/2 (r + 1)) of the tile, both head-dim boxes
-            const void* map = ks.in_b ? &tm_kb : &tm_ka;
-            for (int ch = 0; ch < kQBoxes; ++ch)
-              tma_load_2d_pair(dst + ch * kKBox, map, full, head * DG + ch * 64,
-                               ks.row + (kBN / 2) * static_cast<int>(rank));
-          }
-          if (v8) {  // E4M3 V^T rows d in [64 r, 64 r + 64), all 128 keys
-            tma_load_2d_pair(dst + kKHalf, &tm_vb, full, vs.row, head * D + 64 * static_cast<int>(rank));
-          } else if (vj >= 0 && v_here) {  // head-dim columns [64 r, 64 r + 64) of all kBN keys
-            const void* map = vs.in_b ? &tm_vb : &tm_va;
-            tma_load_2d_pair(dst + kKHalf, map, full, head * DG + 64 * static_cast<int>(rank), vs.row);
-          }
+          const int k = n_pub, s = k % tc2::kItemSlots;
+          if (k >= tc2::kItemSlots &&
+              !wait_cl(bar(L::kItemEmpty + s), static_cast<uint32_t>(k / tc2::kItemSlots - 1) & 1u, ctl, 21))
+            return false;
+          // (with the item's Q buffer, for the epilogue)
+          const uint4 lo = make_uint4(pub_task.q_row0, pub_task.q_rows | (pub_q & 1) << 16, pub_task.a_row0, pub_task.a_len);
+          const uint4 hi = make_uint4(pub_task.b_row0, pub_task.b_len, pub_head, pub_task.part);
+          const uint32_t peer = mapa_shared(ring_slot(k), 1);
+          st_shared_v4(ring_slot(k), lo);
+          st_shared_v4(ring_slot(k) + 16u, hi);
+          st_cluster_v4(peer, lo);
+          st_cluster_v4(peer + 16u, hi);
+          mbar_arrive(bar(L::kItemFull + s));
+          mbar_arrive_release_cluster(mapa_shared(bar(L::kItemFull + s), 1));
+          pub_end = pub_head < 0;
+          if (pub_task.a_len + pub_task.b_len > 0) ++pub_q;
+          ++n_pub;
         }
-        ++g;
+        pub_step = pub_step == 2 ? 0 : pub_step + 1;
         return true;
       };
-      for (int k = 0;; ++k) {
-        const int item = !dyn ? static_item(k) : leader ? publish_item(k) : take_item(k, 18);
-        if (item == -2) goto producer_done;
-        if (item < 0) break;
-        decode_item(args, item, tk, head);
-        const int nkv = tc2::n_key_tiles<kBN>(tk, na);
-        if (nkv == 0) continue;
-        {  // this CTA's 128 query rows into Q buffer qi % 2
-          const int b = qi & 1;
+      // The K side: item k_item - 1, of which K tiles [0, kj) are loaded.
+      Task kt{};
+      int k_item = 0, kj = 0, k_na = 0, k_nkv = 0, qi = 0;
+      bool k_end = false;
+      // The V side: item v_item - 1, tile vj of it is next; G its group of S_1.
+      Task vt{};
+      int v_item = 0, vj = 0, v_na = 0, v_nkv = 0, G = 0;
+      int done = -1;  // groups up to this one are known to be complete
+#pragma unroll 1
+      for (int t = -2;; ++t) {  // V_t (from t = 0 on), then K_t+2
+        if (t >= 0) {
+          while (vj == v_nkv) {  // the next item (the K side has passed it, so it is in the ring)
+            G += v_nkv > 0 || v_item == 0 ? v_nkv + 1 : 0;
+            vt = ring_read(v_item);
+            if (!leader) ring_done(v_item);
+            ++v_item;
+            vj = v_nkv = 0;
+            if (vt.head < 0) break;
+            v_nkv = tc2::n_key_tiles<kBN>(vt, v_na);
+          }
+          if (vt.head < 0) break;
+          // The slots of V_t and K_t+2 are free once the P.V of tile t - kStages
+          // and the S of tile t + 2 - kStages are complete.  Both hold after the
+          // group below, which lies at most four groups before the first that
+          // needs V_t: pair_done's phase of it cannot have passed unseen.
+          const int g = kStages == 3 ? (vj == 0 ? G - 3 : G + vj - 2) : (kF8 && vj == 2 ? G : G + vj - 3);
+          if (g > done) {
+            if (!wait_one(bar(L::kPairDone + (g & 3)), group_parity(g), ctl, 2)) break;
+            done = g;
+          }
+          const int slot = slot_of(t);
+          const TileSrc vs = tc2::tile_src<kBN>(vt, v_na, vj);
+          const bool v8 = kF8 && vs.in_b;
+          const bool v_here = DG == D || rank == 0;  // at head dim 64 only the first CTA loads V
+          const uint32_t vb = v8 ? kVHalf8 : kVHalf;
+          const uint32_t dst = base + L::kRing + static_cast<uint32_t>(slot) * kStage + kKHalf;
+          const uint32_t full = lbar(L::kVFull + slot);
+          if (leader) mbar_arrive_expect_tx(bar(L::kVFull + slot), (DG == D ? 2 : 1) * vb);
+          ++n_ring[kStages + slot];
+          own_bytes[kStages + slot] = v_here ? vb : 0u;
+          other_bytes[kStages + slot] = DG == D || rank == 1 ? vb : 0u;
+          // E4M3: V^T rows d in [64 r, 64 r + 64), all 128 keys; bf16: head-dim
+          // columns [64 r, 64 r + 64) of all kBN keys
+          if (v_here) {
+            const int d0 = vt.head * DG + 64 * static_cast<int>(rank);
+            tma_load_2d_pair(dst, vs.in_b ? &tm_vb : &tm_va, full, v8 ? vs.row : d0, v8 ? d0 : vs.row);
+          }
+          ++vj;
+        }
+        // the K side's next item, once its tiles are loaded; the leader chooses
+        // the item after it from its last tiles on, one step per tile
+        for (;;) {
+          const bool need = !k_end && kj == k_nkv;
+          bool more = leader && !pub_end && n_pub <= k_item && kj + 3 >= k_nkv;
+          while (more) {
+            if (!pub_advance()) goto producer_done;
+            more = need && n_pub <= k_item;
+          }
+          if (!need) break;
+          if (!ring_wait(k_item, 18)) goto producer_done;
+          kt = ring_read(k_item++);
+          k_end = kt.head < 0;
+          if (k_end) break;
+          k_nkv = tc2::n_key_tiles<kBN>(kt, k_na);
+          kj = 0;
+          if (k_nkv == 0) continue;
+          const int b = qi & 1;  // its query rows into Q buffer qi % 2
           const uint32_t n = static_cast<uint32_t>(qi >> 1);
           if (!wait_one(bar(L::kQEmpty + b), (n & 1u) ^ 1u, ctl, 1)) goto producer_done;
           if (leader) mbar_arrive_expect_tx(bar(L::kQFull + b), 2 * kQBoxes * kBoxBytes);
           ++n_q[b];
           const uint32_t qfull = lbar(L::kQFull + b);
           for (int ch = 0; ch < kQBoxes; ++ch)
-            tma_load_2d_pair(base + L::kQ + b * kQTile + ch * kBoxBytes, &tm_q, qfull, head * DG + ch * 64,
-                             tk.q_row0 + 128 * static_cast<int>(rank));
+            tma_load_2d_pair(base + L::kQ + b * kQTile + ch * kBoxBytes, &tm_q, qfull, kt.head * DG + ch * 64,
+                             kt.q_row0 + 128 * static_cast<int>(rank));
+          ++qi;
+          break;
         }
-        if (!load_stage(0, -1)) goto producer_done;
-        if (!load_stage(nkv > 1 ? 1 : -1, -1)) goto producer_done;
-        for (int j = 0; j < nkv; ++j)
-          if (!load_stage(j + 2 < nkv ? j + 2 : -1, j)) goto producer_done;
-        ++qi;
+        if (k_end) continue;
+        const int slot = slot_of(t + 2);
+        const TileSrc ks = tc2::tile_src<kBN>(kt, k_na, kj);
+        const bool k8 = kF8 && ks.in_b;
+        const uint32_t kb = k8 ? kKHalf8 : kKBox * kQBoxes;  // each CTA's bytes
+        if (k8) {
+          // this CTA's softmax warps read the cached tile's scales from ring slot
+          // si % kScaleSlots; the slot's previous tile must have been read
+          const int sl = si % tc2::kScaleSlots, use = si / tc2::kScaleSlots;
+          if (use > 0 && !wait_one(bar(L::kScaleEmpty + sl), static_cast<uint32_t>(use - 1) & 1u, ctl, 16)) break;
+          mbar_arrive_expect_tx(bar(L::kScaleFull + sl), 16u);
+          scale_armed[sl] = use & 1;
+          bulk_load(base + L::kScales + 16u * static_cast<uint32_t>(sl),
+                    args.b_scales + ((kt.b_row0 >> 7) + (kj - k_na)) * args.num_heads + kt.head, 16u,
+                    bar(L::kScaleFull + sl));
+          ++si;
+        }
+        ++kj;
+        if (skip_next) {  // fault injection: the leader never arms or loads this tile
+          skip_next = false;
+          continue;
+        }
+        const uint32_t dst = base + L::kRing + static_cast<uint32_t>(slot) * kStage;
+        const uint32_t full = lbar(L::kKFull + slot);
+        if (leader) mbar_arrive_expect_tx(bar(L::kKFull + slot), 2 * kb);
+        ++n_ring[slot];
+        own_bytes[slot] = kb;
+        other_bytes[slot] = kb;
+        // E4M3: keys [64 r, 64 r + 64), one box of 64 rows x 128 bytes; bf16: keys
+        // [kBN/2 r, kBN/2 (r + 1)) of the tile, a box per 64 head-dim columns
+        const void* map = ks.in_b ? &tm_kb : &tm_ka;
+        const int row = ks.row + (kBN / 2) * static_cast<int>(rank);
+        tma_load_2d_pair(dst, map, full, kt.head * DG, row);
+        if (kQBoxes == 2 && !k8) tma_load_2d_pair(dst + kKBox, map, full, kt.head * DG + 64, row);
       }
     producer_done:
       // the scale ring's barriers are this CTA's own
       for (int s = 0; s < tc2::kScaleSlots; ++s)
         if (scale_armed[s] >= 0) drain_one(bar(L::kScaleFull + s), static_cast<uint32_t>(scale_armed[s]), args.timeout_ns);
-      // stage and Q loads of both CTAs complete on the leader's barriers: record
+      // K, V and Q loads of both CTAs complete on the leader's barriers: record
       // this CTA's loads in the leader's shared memory, where the leader
       // settles and drains them after the teardown's first cluster barrier
       const uint32_t rec = mapa_shared(base + L::kLoadRec + rank * (L::kRecWords * 4u), 0);
-      for (int s = 0; s < kStages; ++s) {
-        st_cluster_u32(rec + 4u * s, static_cast<uint32_t>(n_stage[s]));
-        st_cluster_u32(rec + 4u * (kStages + s), own_bytes[s]);
-        st_cluster_u32(rec + 4u * (2 * kStages + s), other_bytes[s]);
+      for (int s = 0; s < L::kRings; ++s) {
+        st_cluster_u32(rec + 4u * s, static_cast<uint32_t>(n_ring[s]));
+        st_cluster_u32(rec + 4u * (L::kRings + s), own_bytes[s]);
+        st_cluster_u32(rec + 4u * (2 * L::kRings + s), other_bytes[s]);
       }
-      st_cluster_u32(rec + 4u * (3 * kStages), static_cast<uint32_t>(n_q[0]));
-      st_cluster_u32(rec + 4u * (3 * kStages + 1), static_cast<uint32_t>(n_q[1]));
+      st_cluster_u32(rec + 4u * (3 * L::kRings), static_cast<uint32_t>(n_q[0]));
+      st_cluster_u32(rec + 4u * (3 * L::kRings + 1), static_cast<uint32_t>(n_q[1]));
     }
     __syncwarp();
   } else if (warp == Cfg::kMmaWarp) {
     // ------------------------------------------------------------ MMA warp (leader)
     if (leader) {
-      // descriptors of stage 0 (stage s: + s * kStage / 16) and of Q buffer 0
+      // descriptors of ring slot 0 (slot s: + s * kStage / 16) and of Q buffer 0
       const uint64_t kd0 = sdesc_sw128(base + L::kRing, 16, 1024);
       const uint64_t vd0 = sdesc_sw128(base + L::kRing + kKHalf, Cfg::kVHalf, 1024);
       const uint64_t qdesc0 = sdesc_sw128(base + L::kQ, 16, 1024);
@@ -530,116 +619,124 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         return (static_cast<uint32_t>(kk >> 2) * kKBox + static_cast<uint32_t>(kk & 3) * 32u) >> 4;
       };
       bool issued = false;
-      int g = 0, t0 = 0, qi = 0;
-      const volatile int* gate_item = reinterpret_cast<const volatile int*>(base_ptr + L::kGateItem);
-      for (;;) {
-        // the gate warp names the next item with key tiles at this handshake;
-        // none left (or a failed wait) ends both warps
-        if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
-        Task tk;
-        int head, na;
-        decode_item(args, *gate_item, tk, head);
-        const int nkv = tc2::n_key_tiles<kBN>(tk, na);
-        const int qb = qi & 1;
-        const uint64_t qd = qdesc0 + ((static_cast<uint32_t>(qb) * kQTile) >> 4);
-        // groups G, G + 1: S_0, S_1 (the gate warp has seen the Q tile and stage g land)
-        for (int n = 0; n < 2; ++n, ++g) {
-          if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
-          const int slot = stage_of(g);
-          if (lane == 0) {
-            if (n < nkv) {
-              tc_fence_after();
-              const uint64_t kd = kd0 + static_cast<uint64_t>(slot) * (kStage >> 4);
-              const uint32_t d_s = tmem + kColS + static_cast<uint32_t>((t0 + n) & 1) * kBN;
-              if (kF8 && n >= na) {
+      // Groups: the first item's S_0; then per item S_1 (group G), and P_j V_j
+      // with S_j+2 (group G + 1 + j), where S_nkv is the next item's S_0 if that
+      // may be issued ahead (inside this item).  The gate warp names the next
+      // item at the handshake of that group, or of S_1 when nkv = 1 (item q in
+      // entry q % 2: key tiles, 0 if none is left, those of range A, whether S_0
+      // goes ahead).
+      auto slot_k = [&](int t) -> uint64_t { return kd0 + static_cast<uint64_t>(slot_of(t)) * (kStage >> 4); };
+      auto issue_s = [&](uint32_t d_s, uint64_t qd, uint64_t kd, bool s8) {
+        if (kF8 && s8) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                  tc2_mma_ss_f8(d_s, q8d + ((32u * kk) >> 4), kd + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : 0u);
-              } else {
+          for (int kk = 0; kk < 4; ++kk)
+            tc2_mma_ss_f8(d_s, q8d + ((32u * kk) >> 4), kd + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : 0u);
+        } else {
 #pragma unroll
-                for (int kk = 0; kk < DG / 16; ++kk)
-                  tc2_mma_ss(d_s, qd + q_off(kk), kd + k_off(kk), kIdescS, kk > 0 ? 1u : 0u);
-              }
-              if (n == nkv - 1) tc2_commit_mc(bar(L::kQEmpty + qb), 3);
-            }
-            tc2_commit_mc(bar(L::kPairDone + (g & 3)), 3);
-          }
-          issued = true;
-          __syncwarp();
+          for (int kk = 0; kk < DG / 16; ++kk)
+            tc2_mma_ss(d_s, qd + q_off(kk), kd + k_off(kk), kIdescS, kk > 0 ? 1u : 0u);
         }
-        // groups G + 2 + j: P_j V_j (+ S_j+2) (the gate warp has seen P_t, which
-        // also covers this group's stage and the previous item's O reads)
-        for (int j = 0; j < nkv; ++j, ++g) {
-          if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
-          const int t = t0 + j;
-          const int slot = stage_of(g);
-          const uint64_t soff = static_cast<uint64_t>(slot) * (kStage >> 4);
-          const uint64_t vd = vd0 + soff;
-          const uint32_t a_p = tmem + kColP + static_cast<uint32_t>(t & 1) * kPStride;
-          const uint32_t acc0 = j > 0 ? 1u : 0u;
-          if constexpr (kPSplit > 0) {  // P's first chunks
+      };
+      const volatile int* gate_item = reinterpret_cast<const volatile int*>(base_ptr + L::kGateItem);
+      int nkv = 0, na = 0, ahead = 1, nkv_next = 0, na_next = 0, ahead_next = 1;
+      int g = 0, t0 = 0, qi = -1;
+      auto named = [&]() {
+        const volatile int* n = gate_item + 4 * ((qi + 1) & 1);
+        nkv_next = __shfl_sync(0xffffffffu, n[0], 0);
+        if (kF8) na_next = __shfl_sync(0xffffffffu, n[1], 0), ahead_next = __shfl_sync(0xffffffffu, n[2], 0);
+      };
+      // steps without P.V: S_j+2 for j = -2 (the first item's S_0) and j = -1
+      for (int j = -2;;) {
+        if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
+        issued = true;
+        bool s_on = j + 2 < nkv, s_next = false;
+        if (j + 2 == nkv) {
+          named();
+          s_on = s_next = nkv_next > 0 && ahead_next;
+        }
+        if (lane == 0) {
+          tc_fence_after();
+          const int q = qi + (s_next ? 1 : 0);
+          const uint64_t qd = qdesc0 + ((static_cast<uint32_t>(q & 1) * kQTile) >> 4);
+          if (kF8 && j == -1 && !ahead) {  // an S_0 of a cached tile, not issued ahead
+            issue_s(tmem + kColS + static_cast<uint32_t>(t0 & 1) * kBN, qd, slot_k(t0), true);
+            if (nkv == 1) tc2_commit_mc(bar(L::kQEmpty + (qi & 1)), 3);
+          }
+          if (s_on) {
+            issue_s(tmem + kColS + static_cast<uint32_t>((t0 + j) & 1) * kBN, qd, slot_k(t0 + j + 2),
+                    kF8 && !s_next && j + 2 >= na);
+            if (s_next ? nkv_next == 1 : j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (q & 1)), 3);
+          }
+          tc2_commit_mc(bar(L::kPairDone + (g & 3)), 3);
+        }
+        __syncwarp();
+        ++g;
+        if (j == -2) goto next_item;
+        {
+          const uint64_t qd = qdesc0 + ((static_cast<uint32_t>(qi & 1) * kQTile) >> 4);
+          // descriptors and buffers of step j, advanced after each step
+          uint32_t vslot = static_cast<uint32_t>(slot_of(t0)), odd = static_cast<uint32_t>(t0 & 1);
+          uint64_t vd = vd0 + static_cast<uint64_t>(vslot) * (kStage >> 4), kd = slot_k(t0 + 2);
+          uint32_t a_p = tmem + kColP + odd * kPStride, d_s = tmem + kColS + odd * kBN, acc0 = 0;
+          for (j = 0; j < nkv; ++j, ++g) {
+            if (kPSplit > 0) {  // P's first chunks
+              if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
+              if (lane == 0) {
+                tc_fence_after();
+#pragma unroll
+                for (int kk = 0; kk < 2 * kPSplit; ++kk)
+                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+              }
+              __syncwarp();
+            }
+            if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
+            if (j + 2 == nkv) named();
             if (lane == 0) {
               tc_fence_after();
-#pragma unroll
-              for (int kk = 0; kk < 2 * kPSplit; ++kk)
-                tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
-            }
-            issued = true;
-            __syncwarp();
-            if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
-          }
-          if (lane == 0) {
-            tc_fence_after();
-            const bool pv8 = kF8 && j >= na;      // P_j V_j on E4M3 operands
-            const bool s8 = kF8 && j + 2 >= na;   // S_j+2 on E4M3 operands
-            const uint64_t vd8 = vd80 + soff;
-            if (j + 2 < nkv) {
-              const uint64_t kd = kd0 + soff;
-              const uint32_t d_s = tmem + kColS + static_cast<uint32_t>(t & 1) * kBN;
-              if (!s8 && Cfg::kPOverS) {
-                // S_j+2 overwrites P_j: every P.V MMA of the group goes first
+              // P.V first: with P over S, the S overwrites P_j
+              if (!kF8 && j + 2 < nkv) {
 #pragma unroll
                 for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
                   tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+                issue_s(d_s, qd, kd, false);
+                if (j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (qi & 1)), 3);
+              } else {
+                if (kF8 && j >= na) {
+                  const uint64_t vd8 = vd + (vd80 - vd0);
 #pragma unroll
-                for (int kk = 0; kk < DG / 16; ++kk)
-                  tc2_mma_ss(d_s, qd + q_off(kk), kd + k_off(kk), kIdescS, kk > 0 ? 1u : 0u);
-              } else if (!s8) {
+                  for (int kk = 0; kk < 4; ++kk)
+                    tc2_mma_ts_f8(tmem + kColO, a_p + 8u * kk, vd8 + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : acc0);
+                } else {
 #pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
-                  if (kk < DG / 16) tc2_mma_ss(d_s, qd + q_off(kk), kd + k_off(kk), kIdescS, kk > 0 ? 1u : 0u);
+                  for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
+                    tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
                 }
-              } else if (pv8) {
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                  tc2_mma_ts_f8(tmem + kColO, a_p + 8u * kk, vd8 + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : acc0);
-                  tc2_mma_ss_f8(d_s, q8d + ((32u * kk) >> 4), kd + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : 0u);
-                }
-              } else {  // the last live tiles' P.V beside the first cached tiles' S
-#pragma unroll
-                for (int kk = 0; kk < 8; ++kk) {
-                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
-                  if (kk < 4)
-                    tc2_mma_ss_f8(d_s, q8d + ((32u * kk) >> 4), kd + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : 0u);
+                const bool s_next = j + 2 == nkv;
+                if (j + 2 < nkv || (s_next && nkv_next > 0 && ahead_next)) {
+                  const int q = qi + (s_next ? 1 : 0);
+                  issue_s(d_s, qdesc0 + ((static_cast<uint32_t>(q & 1) * kQTile) >> 4), kd, kF8 && !s_next && j + 2 >= na);
+                  if (s_next ? nkv_next == 1 : j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (q & 1)), 3);
                 }
               }
-              if (j + 2 == nkv - 1) tc2_commit_mc(bar(L::kQEmpty + qb), 3);
-            } else if (pv8) {
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                tc2_mma_ts_f8(tmem + kColO, a_p + 8u * kk, vd8 + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : acc0);
-            } else {
-#pragma unroll
-              for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
-                tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+              tc2_commit_mc(bar(L::kPairDone + (g & 3)), 3);
             }
-            tc2_commit_mc(bar(L::kPairDone + (g & 3)), 3);
+            __syncwarp();
+            // K_t+3's slot: kStages 3: V_t's; 4: the one before it
+            kd = kStages == 3 ? kd0 + (vd - vd0) : kd == kd0 + 3ull * (kStage >> 4) ? kd0 : kd + (kStage >> 4);
+            vd = vslot == kStages - 1 ? vd0 : vd + (kStage >> 4);
+            vslot = vslot == kStages - 1 ? 0u : vslot + 1u;
+            odd ^= 1u;
+            a_p = tmem + kColP + odd * kPStride;
+            d_s = tmem + kColS + odd * kBN;
+            acc0 = 1;
           }
-          __syncwarp();
         }
+      next_item:
+        if (nkv_next == 0) break;
         t0 += nkv;
         ++qi;
+        nkv = nkv_next, na = na_next, ahead = ahead_next;
+        j = -1;
       }
     mma_done:
       if (issued && lane == 0) {  // every MMA must finish before TMEM is freed
@@ -653,44 +750,61 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     // The same group sequence as the MMA warp; every wait is bounded, and a
     // failed wait is passed on through the handshake, after which both leave.
     if (leader) {
-      int g = 0, t0 = 0, qi = 0, q8i = 0;
       volatile int* gate_item = reinterpret_cast<volatile int*>(base_ptr + L::kGateItem);
-      for (int k = 0;; ++k) {
-        const int item = take_item_warp(k, 19);
-        Task tk;
-        int head = 0, na = 0, nkv = 0;
-        if (item >= 0) {
-          decode_item(args, item, tk, head);
-          nkv = tc2::n_key_tiles<kBN>(tk, na);
-          if (nkv == 0) continue;
+      auto wait_k = [&](int t) -> bool { return wait_cl_warp(bar(L::kKFull + slot_of(t)), slot_parity(t), ctl, 4); };
+      // the steps of the MMA warp (see there)
+      int nkv = -1, na = 0, nkv_next = 0, na_next = 0, k = 0, q8i = 0;
+#pragma unroll 1
+      for (int t0 = 0, qi = -1, j = -2;;) {
+        const int t = t0 + j;
+        bool ok = true;
+        bool k_wait = j + 2 < nkv;
+        if (j + 2 == max(nkv, 0)) {  // name the next item with keys
+          for (;;) {
+            ok = ok && __all_sync(0xffffffffu, ring_wait(k, 19));
+            if (!ok) break;
+            const Task tk = ring_read(k);
+            __syncwarp();
+            if (lane == 0) ring_done(k);
+            ++k;
+            nkv_next = tk.head < 0 ? 0 : tc2::n_key_tiles<kBN>(tk, na_next);
+            if (tk.head < 0 || nkv_next > 0) break;
+          }
+          if (lane == 0) {
+            volatile int* named = gate_item + 4 * ((qi + 1) & 1);
+            named[0] = nkv_next;
+            named[1] = na_next;
+            // on an E4M3 cache an S_0 of a cached tile cannot go ahead: its Q
+            // tile is written only after the item before it is done
+            named[2] = kF8 && na_next == 0 ? 0 : 1;
+          }
+          __syncwarp();
+          k_wait = nkv_next > 0;
+          if (k_wait)
+            ok = ok && wait_cl_warp(bar(L::kQFull + ((qi + 1) & 1)), static_cast<uint32_t>((qi + 1) >> 1) & 1u, ctl, 3);
         }
-        // the MMA warp takes the item from here; the end of the list, or a
-        // failed wait, ends both warps
-        if (lane == 0) *gate_item = item;
-        if (bar_red_or(tc2::kGateBarrier, 64, item < 0)) goto gate_done;
+        if (k_wait) ok = ok && wait_k(t + 2);
         // the first cached tile's S also needs the E4M3 Q tile of both CTAs
-        const bool q8 = kF8 && nkv > na;
-        const uint32_t q8_parity = static_cast<uint32_t>(q8i) & 1u;
-        bool ok = wait_cl_warp(bar(L::kQFull + (qi & 1)), static_cast<uint32_t>(qi >> 1) & 1u, ctl, 3);
-        for (int n = 0; n < 2; ++n, ++g) {
-          ok = ok && wait_cl_warp(bar(L::kStageFull + stage_of(g)), stage_parity(g), ctl, 4);
-          if (q8 && n == na) ok = ok && wait_cl_warp(bar(L::kQ8Full), q8_parity, ctl, 14);
-          if (bar_red_or(tc2::kGateBarrier, 64, !ok)) goto gate_done;
+        if (kF8 && nkv > na && (j + 2 == na || (j == -1 && na == 0))) {
+          ok = ok && wait_cl_warp(bar(L::kQ8Full), static_cast<uint32_t>(q8i) & 1u, ctl, 14);
+          ++q8i;
         }
-        for (int j = 0; j < nkv; ++j, ++g) {
-          const int t = t0 + j;
+        if (j >= 0) {
+          ok = ok && wait_cl_warp(bar(L::kVFull + slot_of(t)), slot_parity(t), ctl, 13);
           if constexpr (kPSplit > 0) {
-            ok = wait_cl_warp(bar(L::kStageFull + stage_of(g)), stage_parity(g), ctl, 13);
             ok = ok && wait_cl_warp(bar(L::kPHalf + (t & 1)), static_cast<uint32_t>(t >> 1) & 1u, ctl, 22);
             if (bar_red_or(tc2::kGateBarrier, 64, !ok)) goto gate_done;
           }
-          ok = wait_cl_warp(bar(L::kPFull + (t & 1)), static_cast<uint32_t>(t >> 1) & 1u, ctl, 7);
-          if (q8 && j + 2 == na) ok = ok && wait_cl_warp(bar(L::kQ8Full), q8_parity, ctl, 14);
-          if (bar_red_or(tc2::kGateBarrier, 64, !ok)) goto gate_done;
+          ok = ok && wait_cl_warp(bar(L::kPFull + (t & 1)), static_cast<uint32_t>(t >> 1) & 1u, ctl, 7);
         }
-        t0 += nkv;
-        ++qi;
-        if (q8) ++q8i;
+        if (bar_red_or(tc2::kGateBarrier, 64, !ok)) goto gate_done;
+        if (++j >= nkv) {
+          if (nkv_next == 0) break;
+          t0 += max(nkv, 0);
+          ++qi;
+          nkv = nkv_next, na = na_next;
+          j = -1;
+        }
       }
     gate_done:;
     }
@@ -715,7 +829,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     const f32x2 sl2x2 = make_f32x2(sl2, sl2);
     float* lx = reinterpret_cast<float*>(base_ptr + L::kLX);  // [2][128] partial row sums (kH = 2)
     int t = 0;     // tiles of earlier items
-    int G = 0;     // first group of the item
+    int G = 1;     // the item's group of S_1 (S_j: ready after group G + j - 1; P_j V_j: group G + 1 + j)
     int n_lx = 0;  // row-sum exchanges so far (kH = 2)
     int si = 0;    // cached tiles read from the scale ring so far
     // wait until group g is complete (both CTAs see the multicast commit)
@@ -723,23 +837,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       return wait_cl_warp(bar(L::kPairDone + (g & 3)), group_parity(g), ctl, where);
     };
     for (int k = 0;; ++k) {
-      const int item = take_item_warp(k, 20);
-      if (item == -2) goto softmax_done;
-      if (item < 0) break;
-      Task tk;
-      int head;
-      decode_item(args, item, tk, head);
+      if (!__all_sync(0xffffffffu, ring_wait(k, 20))) goto softmax_done;
+      const Task tk = ring_read(k);
+      const int head = tk.head;
+      if (head < 0) break;
       int na;
       const int nkv = tc2::n_key_tiles<kBN>(tk, na);
-      const bool row_ok = prow < tk.q_rows;
+      const bool row_ok = prow < (tk.q_rows & 0xFFFF);
       const int64_t grow = static_cast<int64_t>(tk.q_row0) + prow;
-      __nv_bfloat16* orow = args.out + grow * args.row_stride + static_cast<int64_t>(head) * DG + ocol0;
       if (nkv == 0) {
         if (row_ok) {
+          __nv_bfloat16* orow = args.out + grow * args.row_stride + static_cast<int64_t>(head) * DG + ocol0;
           uint4 z = make_uint4(0, 0, 0, 0);
           for (int c = 0; c < kOC / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = z;
           if (args.lse && hh == 0) args.lse[grow * args.num_heads + head] = -INFINITY;
         }
+        __syncwarp();
+        if (lane == 0) ring_done(k);
         continue;
       }
       float m_run = 0.f, l_run = 0.f;
@@ -816,8 +930,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           wshift = 0.f;
           lscale = nz ? s_ref * sc.w : 1.f;  // 2^-delta
         }
-        // S_j is ready and P buffer b is free once group G + j is complete
-        if (!wait_group(G + j, 8)) goto softmax_done;
+        // S_j is ready and P buffer b is free once group G + j - 1 is complete
+        // (one later for an S_0 that was not issued ahead)
+        if (!wait_group(G + j - (kF8 && j == 0 && na == 0 ? 0 : 1), 8)) goto softmax_done;
         tc_fence_after();
         const uint32_t t_s = tmem + lane_off + kColS + static_cast<uint32_t>(kBN) * b;
         // Keys past the end of the range: -inf, written over their scores in
@@ -865,9 +980,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
             m_raw = fmax3(mx[0], mx[1], fmaxf(mx[2], mx[3]));
         }
         // rescale this row's O columns and l for a new running maximum m_new (O
-        // must first hold P_j-1 V_j-1: group G + j + 1 complete)
+        // must first hold P_j-1 V_j-1: group G + j complete)
         auto rescale = [&](float m_new) -> bool {
-          if (!wait_group(G + j + 1, 9)) return false;
+          if (!wait_group(G + j, 9)) return false;
           tc_fence_after();
           const float alpha = ex2_approx(m_run - m_new);
           const f32x2 alpha2 = make_f32x2(alpha, alpha);
@@ -958,29 +1073,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         }
         const float l_tile = write_p();
         l_run += kF8 ? l_tile * lscale : l_tile;
-        // the MMA thread waits only for P: the leader's warp 0 first makes
-        // sure that the stage of P_j V_j's group (G + j + 2) has landed
-        if (kPSplit == 0 && leader && warp == 0 &&
-            !wait_warp(bar(L::kStageFull + stage_of(G + j + 2)), stage_parity(G + j + 2), ctl, 13))
-          goto softmax_done;
         p_arrive(L::kPFull + b);
       }
       {
-        // the row's place: the bf16 kernels read it again from the work list, so
-        // that it is not kept live through the tile loop
-        bool e_row_ok = row_ok;
-        int64_t e_grow = grow;
-        __nv_bfloat16* e_orow = orow;
-        int e_head = head, e_part = tk.part;
-        if constexpr (!kF8) {
-          Task et;
-          decode_item(args, item, et, e_head);
-          e_row_ok = prow < et.q_rows;
-          e_grow = static_cast<int64_t>(et.q_row0) + prow;
-          e_orow = args.out + e_grow * args.row_stride + static_cast<int64_t>(e_head) * DG + ocol0;
-          e_part = et.part;
-        }
-        if (!wait_group(G + nkv + 1, 10)) goto softmax_done;  // the item's last group
+        // the row's place is read again from the item ring, so that it is not
+        // kept live through the tile loop
+        const Task et = ring_read(k);
+        const int e_rows = et.q_rows & 0xFFFF, e_qb = et.q_rows >> 16, e_head = et.head, e_part = et.part;
+        const bool e_row_ok = prow < e_rows;
+        const int64_t e_grow = static_cast<int64_t>(et.q_row0) + prow;
+        __syncwarp();
+        if (lane == 0) ring_done(k);
+        if (!wait_group(G + nkv, 10)) goto softmax_done;  // the item's last group
         tc_fence_after();
         float l_tot = l_run;
         if constexpr (kH == 2) {
@@ -995,9 +1099,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         const float inv_l = kF8 ? s_ref / l_tot : 1.0f / l_tot;
         const uint32_t t_o = tmem + lane_off + kColO + static_cast<uint32_t>(ocol0);
         if (e_part > 0) {
-          // a part of a split item: O / l in fp32 and m + log l to its workspace slot
-          const int64_t prow_ws = static_cast<int64_t>(e_part - 1) * args.rows_per_task + prow;
-          float4* dst = reinterpret_cast<float4*>(args.part_o + prow_ws * DG + ocol0);
+          // a part of a split item: O / l in fp32 and m + log l to its workspace
+          // slot, [D / 4][rows_per_task] float4, so that a warp's 32 rows of four
+          // columns are one run of 512 bytes
+          const int64_t slot = e_part - 1;
+          float4* dst = reinterpret_cast<float4*>(args.part_o) + (slot * (DG / 4) + ocol0 / 4) * args.rows_per_task + prow;
 #pragma unroll
           for (int cc = 0; cc < kOC / 32; ++cc) {
             uint32_t o[32];
@@ -1006,40 +1112,66 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
             if (e_row_ok) {
 #pragma unroll
               for (int c = 0; c < 8; ++c)
-                dst[8 * cc + c] = make_float4(__uint_as_float(o[4 * c]) * inv_l, __uint_as_float(o[4 * c + 1]) * inv_l,
-                                              __uint_as_float(o[4 * c + 2]) * inv_l,
-                                              __uint_as_float(o[4 * c + 3]) * inv_l);
+                dst[(8 * cc + c) * args.rows_per_task] =
+                    make_float4(__uint_as_float(o[4 * c]) * inv_l, __uint_as_float(o[4 * c + 1]) * inv_l,
+                                __uint_as_float(o[4 * c + 2]) * inv_l, __uint_as_float(o[4 * c + 3]) * inv_l);
             }
           }
           tc_fence_before();
-          if (e_row_ok && hh == 0) args.part_lse[prow_ws] = (m_run + log2f(l_tot)) * 0.69314718055994530942f;
-          G += nkv + 2;
-          continue;
-        }
-        uint32_t packed[kOC / 2];
+          if (e_row_ok && hh == 0)
+            args.part_lse[slot * args.rows_per_task + prow] = (m_run + log2f(l_tot)) * 0.69314718055994530942f;
+        } else {
+          // O / l as bf16 through the item's Q buffer, which its S no longer
+          // reads: this thread's row in 16-byte chunks (swizzled), then whole
+          // rows to global memory, kNC lanes each.  Stored straight from the
+          // registers a warp's 16 bytes per row touch 32 lines per instruction,
+          // 2048 cycles of the SM's load/store unit per item, which the next
+          // item's softmax waited for.
+          constexpr int kNC = kOC / 8;                       // this thread's chunks of the row
+          constexpr uint32_t kPitch = 16u * kNC * kH;        // bytes of a staged row
+          const uint32_t stage = base + L::kQ + static_cast<uint32_t>(e_qb) * kQTile +
+                                 static_cast<uint32_t>(quarter * 32) * kPitch + static_cast<uint32_t>(hh) * 16u * kNC;
 #pragma unroll
-        for (int cc = 0; cc < kOC / 32; ++cc) {
-          uint32_t o[32];
-          tmem_ld32(t_o + 32u * cc, o);
-          tmem_wait_ld(o);
+          for (int cc = 0; cc < kOC / 32; ++cc) {
+            uint32_t o[32];
+            tmem_ld32(t_o + 32u * cc, o);
+            tmem_wait_ld(o);
 #pragma unroll
-          for (int c = 0; c < 16; ++c)
-            packed[16 * cc + c] =
-                pack_bf16x2(__uint_as_float(o[2 * c]) * inv_l, __uint_as_float(o[2 * c + 1]) * inv_l);
-        }
-        // (the next arrival on p_full, after the next tile's P, tells the MMA
-        // thread that these O reads are done)
-        tc_fence_before();
-        if (e_row_ok) {
-          uint4* dst = reinterpret_cast<uint4*>(e_orow);
+            for (int c = 0; c < 4; ++c) {
+              uint32_t w[4];
 #pragma unroll
-          for (int c = 0; c < kOC / 8; ++c)
-            dst[c] = make_uint4(packed[4 * c], packed[4 * c + 1], packed[4 * c + 2], packed[4 * c + 3]);
-          if (args.lse && hh == 0)
+              for (int e = 0; e < 4; ++e)
+                w[e] = pack_bf16x2(__uint_as_float(o[8 * c + 2 * e]) * inv_l, __uint_as_float(o[8 * c + 2 * e + 1]) * inv_l);
+              st_shared_v4(stage + static_cast<uint32_t>(lane) * kPitch +
+                               ((static_cast<uint32_t>(4 * cc + c) ^ static_cast<uint32_t>(lane & (kNC - 1))) << 4),
+                           make_uint4(w[0], w[1], w[2], w[3]));
+            }
+          }
+          // (the next arrival on p_full, after the next tile's P, tells the MMA
+          // thread that these O reads are done)
+          tc_fence_before();
+          __syncwarp();
+          constexpr int kRows = 32 / kNC;  // rows per instruction
+          const int r0 = lane / kNC, ch = lane % kNC;
+          const int first = 128 * static_cast<int>(rank) + quarter * 32;  // the warp's first row in the item
+          __nv_bfloat16* dst = args.out + (static_cast<int64_t>(et.q_row0) + first) * args.row_stride +
+                               static_cast<int64_t>(e_head) * DG + ocol0 + 8 * ch;
+#pragma unroll 4
+          for (int i = 0; i < kNC; ++i) {
+            const int r = i * kRows + r0;
+            const uint4 v = ld_shared_v4(stage + static_cast<uint32_t>(r) * kPitch +
+                                         (static_cast<uint32_t>(ch ^ (r & (kNC - 1))) << 4));
+            if (first + r < e_rows) *reinterpret_cast<uint4*>(dst + r * args.row_stride) = v;
+          }
+          if (e_row_ok && args.lse && hh == 0)
             args.lse[e_grow * args.num_heads + e_head] = (m_run + log2f(l_tot)) * 0.69314718055994530942f;
         }
+        // the Q buffer is free for the TMA loads of the item after the next
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(L::kQEmpty + e_qb));
       }
-      G += nkv + 2;
+      G += nkv + 1;
     }
   softmax_done:;
   }
@@ -1054,7 +1186,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     tmem_dealloc_pair(tmem, kTmemCols);
   }
   if (leader && warp == Cfg::kProducerWarp && lane == 0) {
-    // Every stage and Q load of either CTA must land before that CTA exits.
+    // Every K, V and Q load of either CTA must land before that CTA exits.
     // The leader arms a phase for both halves before it issues its own, and
     // each CTA issues its half after the same wait; after an abort the two can
     // differ by one phase.  A phase the follower loaded but the leader never
@@ -1074,12 +1206,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       }
       if (mine > 0) drain_one(b, static_cast<uint32_t>(mine - 1) & 1u, args.timeout_ns);
     };
-    for (int s = 0; s < kStages; ++s)
-      settle(bar(L::kStageFull + s), static_cast<int>(rec[s]), static_cast<int>(peer[s]), rec[2 * kStages + s],
-             peer[kStages + s]);
+    for (int s = 0; s < L::kRings; ++s)  // K slots, then V slots
+      settle(bar(L::kKFull + s), static_cast<int>(rec[s]), static_cast<int>(peer[s]), rec[2 * L::kRings + s],
+             peer[L::kRings + s]);
     constexpr uint32_t kQCta = kQBoxes * kBoxBytes;  // each CTA's bytes of a Q load
     for (int b = 0; b < 2; ++b)
-      settle(bar(L::kQFull + b), static_cast<int>(rec[3 * kStages + b]), static_cast<int>(peer[3 * kStages + b]),
+      settle(bar(L::kQFull + b), static_cast<int>(rec[3 * L::kRings + b]), static_cast<int>(peer[3 * L::kRings + b]),
              kQCta, kQCta);
   }
   // the follower leaves only once the leader has seen every load of the pair land

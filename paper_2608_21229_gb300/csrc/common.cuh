@@ -45,7 +45,7 @@ struct AttnArgs {
   float scale_log2;             // softmax_scale * log2(e)
   int32_t rows_per_task;        // 128 or 256 (the mma.sync kernel splits tasks into 64-row CTAs)
   int32_t per_item;             // tasks is a per-item list (Task::head, Task::part used)
-  float* part_o;                // workspace of partial results: [slot][rows_per_task][D] fp32, O / l
+  float* part_o;                // workspace of partial results: [slot][D / 4][rows_per_task][4] fp32, O / l
   float* part_lse;              //                               [slot][rows_per_task] fp32, m + log l
   uint64_t timeout_ns;          // bound of every in-kernel wait
   const float4* b_scales;       // E4M3 key range B: (s_K, s_V, log2 s_V, 1/s_V) per (128-row tile, head), tile-major

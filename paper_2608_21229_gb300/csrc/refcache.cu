@@ -409,7 +409,8 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
   if (copy && (rc = launch_copy(*copy, info, s, true)) != 0) return rc;
   if (il && il->n_jobs > 0) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>((a.rows_per_task + 7) / 8), static_cast<unsigned>(il->n_jobs));
+    cfg.gridDim = dim3(static_cast<unsigned>((a.rows_per_task + rc::kCombineRows - 1) / rc::kCombineRows),
+                       static_cast<unsigned>(il->n_jobs));
     cfg.blockDim = dim3(256, 1, 1);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];

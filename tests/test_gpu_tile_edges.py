@@ -55,3 +55,38 @@ def test_keys_past_the_end_do_not_enter_the_maximum_e4m3(monkeypatch, lengths):
     rcb.set_kernel("tcgen05")
     monkeypatch.setattr(workloads, "live_qkv", lambda *a, **k: live)
     fp8.check_step(fp8.Fp8Run(w, static=static), np.arange(2), statistical=False)
+
+
+#: items of one to four key tiles after one another (an item's first S is issued
+#: inside the item before it, whose last tiles it follows), repeated so that the
+#: ring of items wraps several times on every CTA pair
+SHORT = [(1, 1), (200, 1), (64, 300), (193, 5), (17, 130), (400, 385), (5, 64), (256, 190), (130, 500), (3, 2)]
+
+
+@pytest.mark.parametrize("kernel", ["tcgen05", "tcgen05_k128"])
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_short_items_after_one_another(kernel, head_dim):
+    reqs = tuple(workloads.Request(i % 3, 0, *SHORT[i % len(SHORT)]) for i in range(90))
+    pu.full_compare(pu.GpuRun(workloads.Workload("short_items", 7, head_dim, reqs, 32), kernel=kernel))
+
+
+def test_short_items_after_one_another_e4m3():
+    reqs = tuple(workloads.Request(i % 3, 0, *SHORT[i % len(SHORT)]) for i in range(60))
+    rcb.set_kernel("tcgen05")
+    fp8.check_step(fp8.Fp8Run(workloads.Workload("short_items_fp8", 7, 128, reqs, 33)), np.arange(7), rows_per_request=8,
+                   statistical=False)
+
+
+@pytest.mark.parametrize("head_dim", [64, 128])
+def test_short_items_in_static_order(head_dim):
+    """full_attention_noalloc hands items out in a fixed order: the same bytes as the work counter's."""
+    cu = np.concatenate([[0], np.cumsum([1 + (i * 37) % 420 for i in range(120)])]).tolist()
+    q, k, v = (torch.randn(cu[-1], 5, head_dim, device="cuda", generator=torch.Generator("cuda").manual_seed(s)).to(torch.bfloat16)
+               for s in (1, 2, 3))
+    outs = []
+    for call in (rcb.full_attention, rcb.full_attention_noalloc):
+        o, lse = torch.empty_like(q), torch.empty(cu[-1], 5, device="cuda")
+        call(cu, q, k, v, o, lse)
+        assert rcb.status() == rcb.OK, rcb.last_error()
+        outs.append((o, lse))
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
