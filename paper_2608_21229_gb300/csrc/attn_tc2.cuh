@@ -83,7 +83,7 @@
 //   p_full[t % 2]      one arrival per softmax warp of both CTAs.  Its phase
 //                      for tile t means P_t is in TMEM and every softmax thread
 //                      has finished reading O for the previous item.
-//   p_half[t % 2]      192-key tiles: the same for P's first 32 keys, whose
+//   p_half[t % 2]      192-key tiles: the same for P's first 96 keys, whose
 //                      P.V MMAs are issued while the softmax works on the rest
 //   k_full[s] v_full[s]  the producers' TMA bytes of both CTAs (leader's barriers)
 //   q_full             per Q buffer, once per item
@@ -99,12 +99,18 @@
 // buffer (1536 tensor cycles) cannot start before its softmax is done, and with
 // two S buffers that loop -- S ready, softmax, P, MMAs, next S ready -- set the
 // period: 1880 cycles per tile at 4608 live and 20480 cached rows, 24 heads, of
-// which the MMA thread waited 480 for P.  With the first 32 keys handed over
-// early, their handshake, the V slot's check and the start of the P.V MMAs leave
-// the loop: 1698 cycles per tile, 143 of them waiting.  Larger first pieces are
-// no faster (64 keys 1693, 96 keys 1710, 128 keys 1757 cycles) and slower in
-// time where power sets the clock (interleaved, one run: 32 keys 875 us, 64
-// keys 924, 96 keys 914, one piece 956).
+// which the MMA thread waited 480 for P.  With the first 96 keys handed over
+// early, their handshake and their P.V MMAs leave the loop.  Cycles per tile by
+// the size of the first piece: 32 keys 1743, 64 keys 1700, 96 keys 1697, 128
+// keys 1711 (32 keys measured best while the softmax warps still took 300
+// cycles more per tile than now).  The MMA thread now issues for 1507 of the 1536
+// cycles that a tile's MMAs take and waits 150.
+//
+// The softmax warps are as long in a tile (about 1550 cycles: loads and maximum
+// 215, exponentials and P 1180 of which the exponential unit needs 800, the rest
+// the waits and the loop), so they look at the next S while their last stores of
+// P drain instead of waiting for it afterwards (130 cycles of latency per tile),
+// and find a tile's end from the item's lengths with two instructions.
 //
 // E4M3 cache (kF8): key range B is the quantised reference cache -- K as
 // E4M3 codes [rows_pad, H, 128] and V transposed per head [H, 128, rows_pad],
@@ -166,7 +172,7 @@ struct Cfg {
   static constexpr uint32_t kColO = 384;
   // 32-key chunks of P handed over ahead of the rest (0: P in one piece), see
   // the head of the file
-  static constexpr int kPSplit = kPOverS ? 1 : 0;
+  static constexpr int kPSplit = kPOverS ? 3 : 0;
   static_assert(2 * kBN <= 384 && kColO + kD <= tc::kTmemCols, "tensor-memory layout");
 };
 constexpr int kPairDoneBars = 4;          // pair_done[g % 4]: a waiter for group g holds up group g + 4
@@ -828,6 +834,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     const float sl2 = args.scale_log2;
     const f32x2 sl2x2 = make_f32x2(sl2, sl2);
     float* lx = reinterpret_cast<float*>(base_ptr + L::kLX);  // [2][128] partial row sums (kH = 2)
+    const uint32_t lp = lbar(0);  // the leader's barriers (mapped once)
     int t = 0;     // tiles of earlier items
     int G = 1;     // the item's group of S_1 (S_j: ready after group G + j - 1; P_j V_j: group G + 1 + j)
     int n_lx = 0;  // row-sum exchanges so far (kH = 2)
@@ -906,43 +913,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         s_ref = sc0.y > 0.f ? sc0.y : 1.f;
         l2_ref = sc0.y > 0.f ? sc0.z : 0.f;
       }
+      bool ready = false;  // this tile's S was seen ready at the end of the tile before
       for (int j = 0; j < nkv; ++j, ++t) {
         const int b = t & 1;
-        const TileSrc src = tc2::tile_src<kBN>(tk, na, j);
+        const int valid = (j < na ? tk.a_len : tk.b_len + na * kBN) - j * kBN;  // keys inside the range (>= kBN: all)
         // per-tile constants: u = c * s + shift is the shifted scaled score, the
         // weight written is exp2(u - m + wshift), the tile adds lscale * sum to l
         const bool t8 = kF8 && j >= na;
         float c_t = sl2, shift = 0.f, wshift = -l2_ref, lscale = s_ref;
-        if (t8) {
-          // the producer's ring of tile scales (no global access here: an
-          // ordinary load still in flight would hold up the next P arrival)
-          const int sl = si % tc2::kScaleSlots;
-          if (!wait_warp(bar(L::kScaleFull + sl), static_cast<uint32_t>(si / tc2::kScaleSlots) & 1u, ctl, 17))
-            goto softmax_done;
-          const float4 sc = ld_shared_f4(base + L::kScales + 16u * static_cast<uint32_t>(sl));
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(L::kScaleEmpty + sl));
-          ++si;
-          c_t = fmaxf(c_row * sc.x, 1e-30f);
-          // delta = log2(s_V / s_ref); an all-zero V tile (s_V = 0) takes delta = 0
-          const bool nz = sc.y > 0.f;
-          shift = nz ? sc.z - l2_ref : 0.f;
-          wshift = 0.f;
-          lscale = nz ? s_ref * sc.w : 1.f;  // 2^-delta
-        }
         // S_j is ready and P buffer b is free once group G + j - 1 is complete
         // (one later for an S_0 that was not issued ahead)
-        if (!wait_group(G + j - (kF8 && j == 0 && na == 0 ? 0 : 1), 8)) goto softmax_done;
+        if (!ready && !wait_group(G + j - (kF8 && j == 0 && na == 0 ? 0 : 1), 8)) goto softmax_done;
         tc_fence_after();
         const uint32_t t_s = tmem + lane_off + kColS + static_cast<uint32_t>(kBN) * b;
         // Keys past the end of the range: -inf, written over their scores in
         // tensor memory (a tile with such keys is rare; selects over the loaded
         // columns were 8 KB of code inside the loop, see wait_more).
-        if (src.valid < kBN) {
+        if (valid < kBN) {
           uint32_t inf[16];
 #pragma unroll
           for (int c = 0; c < 16; ++c) inf[c] = 0xFF800000u;
-          int c = src.valid;
+          int c = valid;
 #pragma unroll 1
           for (; c & 15; ++c) tmem_st1(t_s + static_cast<uint32_t>(c), 0xFF800000u);
 #pragma unroll 1
@@ -967,6 +958,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           for (int k = 0; k < kChains; ++k) {
             const uint32_t col = static_cast<uint32_t>(kH == 1 ? 32 * k : (col0 + 32 * k) & (kBN - 1));
             tmem_ld32_max(t_s + col, r[k], mx[k]);
+          }
+          if (t8) {
+            // the producer's ring of tile scales (no global access here: an
+            // ordinary load still in flight would hold up the next P arrival)
+            const int sl = si % tc2::kScaleSlots;
+            if (!wait_warp(bar(L::kScaleFull + sl), static_cast<uint32_t>(si / tc2::kScaleSlots) & 1u, ctl, 17))
+              goto softmax_done;
+            const float4 sc = ld_shared_f4(base + L::kScales + 16u * static_cast<uint32_t>(sl));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(L::kScaleEmpty + sl));
+            ++si;
+            c_t = fmaxf(c_row * sc.x, 1e-30f);
+            // delta = log2(s_V / s_ref); an all-zero V tile (s_V = 0) takes delta = 0
+            const bool nz = sc.y > 0.f;
+            shift = nz ? sc.z - l2_ref : 0.f;
+            wshift = 0.f;
+            lscale = nz ? s_ref * sc.w : 1.f;  // 2^-delta
           }
 #pragma unroll
           for (int k = 0; k < kChains; ++k) tmem_wait_ld(r[k], mx[k]);
@@ -1014,7 +1022,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           tmem_wait_st();
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive_cluster(mapa_shared(bar(which), 0));
+          if (lane == 0) mbar_arrive_cluster(lp + 8u * static_cast<uint32_t>(which));
         };
         auto write_p = [&]() -> float {
           const float bias = (kF8 ? shift + wshift : 0.f) - m_run;
@@ -1073,7 +1081,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         }
         const float l_tile = write_p();
         l_run += kF8 ? l_tile * lscale : l_tile;
+        // a look at the next S, whose latency passes beside the stores of P
+        const bool next_done = j + 1 < nkv && mbar_test_wait(bar(L::kPairDone + ((G + j) & 3)), group_parity(G + j));
         p_arrive(L::kPFull + b);
+        ready = __all_sync(0xffffffffu, next_done);
       }
       {
         // the row's place is read again from the item ring, so that it is not
