@@ -65,16 +65,12 @@
 // went from 5100 to 2700 cycles; step with 1280 live and 2048 cached rows
 // (items of 9 tiles), 24 heads: 62.7 -> 60.7 us.
 //
-// Synchronisation is built so that the MMA thread does as little as possible
-// between its MMAs: a tcgen05.mma blocks its thread until the tensor core
-// takes it, and the tensor core queues almost nothing, so every cycle the
-// MMA thread spends between two groups idles the tensor core.  An mbarrier
-// wait whose result the MMA thread needs costs it far more than a
-// named-barrier handshake, so all mbarrier waits are done by the gate warp:
-// per group, the gate warp waits for what the group needs and then meets the
-// MMA warp at `bar.red.or` (which also carries an abort bit: both warps walk
-// the same group sequence and leave together, so neither can be left waiting);
-// the MMA thread then issues the group and commits once:
+// Synchronisation is built so that the MMA thread waits on nothing itself: all
+// mbarrier waits are done by the gate warp: per group, the gate warp waits for
+// what the group needs and then meets the MMA warp at `bar.red.or` (which also
+// carries an abort bit: both warps walk the same group sequence and leave
+// together, so neither can be left waiting); the MMA thread then issues the group
+// and commits once:
 //   pair_done[g % 4]   one commit per group (multicast to both CTAs): its S
 //                      is in TMEM, its P.V is in O, the ring slots and the P
 //                      buffer it read are free.  Four barriers, so that no
@@ -90,10 +86,12 @@
 //   q_empty            per Q buffer: the item's last S has read it, and the
 //                      epilogue no longer stages O in it
 //   item_full / item_empty  per slot of the item ring
-// The values that MMA operands are computed from (tensor-memory base, warp
-// index, key tiles) pass through a shuffle, which tells the compiler that they
-// are the same in all lanes: operands of tcgen05.mma live in uniform registers,
-// and moving each of them there cost the MMA thread 300 cycles per tile.
+// The MMAs' operands live in uniform registers.  The MMAs are issued under
+// elect.sync, from which the compiler knows that one lane runs (under `lane ==
+// 0` it has to cope with any set of lanes, and a tile's 20 MMAs took 1507 cycles
+// to issue instead of 610, about as long as the tensor core needs for them), and
+// the values the operands are computed from (tensor-memory base, warp index, key
+// tiles) pass through a shuffle, which makes them the same in all lanes.
 //
 // P in two pieces (192-key tiles): a tile's P.V and the S that reuses its
 // buffer (1536 tensor cycles) cannot start before its softmax is done, and with
@@ -102,9 +100,9 @@
 // which the MMA thread waited 480 for P.  With the first 96 keys handed over
 // early, their handshake and their P.V MMAs leave the loop.  Cycles per tile by
 // the size of the first piece: 32 keys 1743, 64 keys 1700, 96 keys 1697, 128
-// keys 1711 (32 keys measured best while the softmax warps still took 300
-// cycles more per tile than now).  The MMA thread now issues for 1507 of the 1536
-// cycles that a tile's MMAs take and waits 150.
+// keys 1711 (with the MMAs under elect.sync 1678, 1635 and 1641 for 64, 96 and
+// 128 keys; 32 keys measured best while the softmax warps still took 300 cycles
+// more per tile than now).
 //
 // The softmax warps are as long in a tile (about 1550 cycles: loads and maximum
 // 215, exponentials and P 1180 of which the exponential unit needs 800, the rest
@@ -660,7 +658,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           named();
           s_on = s_next = nkv_next > 0 && ahead_next;
         }
-        if (lane == 0) {
+        if (elect_one()) {
           tc_fence_after();
           const int q = qi + (s_next ? 1 : 0);
           const uint64_t qd = qdesc0 + ((static_cast<uint32_t>(q & 1) * kQTile) >> 4);
@@ -687,7 +685,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           for (j = 0; j < nkv; ++j, ++g) {
             if (kPSplit > 0) {  // P's first chunks
               if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
-              if (lane == 0) {
+              if (elect_one()) {
                 tc_fence_after();
 #pragma unroll
                 for (int kk = 0; kk < 2 * kPSplit; ++kk)
@@ -697,7 +695,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
             }
             if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
             if (j + 2 == nkv) named();
-            if (lane == 0) {
+            if (elect_one()) {
               tc_fence_after();
               // P.V first: with P over S, the S overwrites P_j
               if (!kF8 && j + 2 < nkv) {

@@ -291,6 +291,17 @@ __device__ __forceinline__ void tc2_commit_mc(uint32_t bar, uint16_t cta_mask) {
       : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+
 // ---------------------------------------------------------------- named barriers
 // Named barrier `id` over `nthreads` threads (whole warps, all lanes of each
 // participating warp execute it); returns the OR of every thread's `pred`.
