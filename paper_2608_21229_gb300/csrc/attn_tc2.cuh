@@ -209,7 +209,8 @@ struct SmemT {
   // head -1: none left); the gate warp passes the MMA warp its item's tiles
   static constexpr uint32_t kItemRing = (kLoadRec + 2 * kRecWords * 4 + 15u) & ~15u;
   static constexpr uint32_t kGateItem = kItemRing + 32 * kItemSlots;  // two of [key tiles, of range A, first S ahead, -]
-  static constexpr uint32_t kUsed = kGateItem + 32;
+  static constexpr uint32_t kPeerAbort = kGateItem + 32;  // the other CTA's abort flag, at teardown
+  static constexpr uint32_t kUsed = kPeerAbort + 4;
   static constexpr uint32_t kMaxDynamic = 232448;
   static constexpr uint32_t kDynamic = kUsed + 1024 < kMaxDynamic ? kUsed + 1024 : kMaxDynamic;
   static_assert(kUsed <= kMaxDynamic, "shared-memory layout too large");
@@ -254,9 +255,9 @@ __device__ __forceinline__ bool wait_cl_warp(uint32_t bar, uint32_t parity, cons
   const bool ok = wait_cl(bar, parity, c, where);
   return __all_sync(0xffffffffu, ok);
 }
-// Work counter [next item, clusters done]: this cluster has finished (every
-// item it took is done or abandoned); the last cluster resets both words for
-// the next launch, which reads them only after this grid has completed.
+// Work counter [next item, clusters done]: this cluster takes no more items; the
+// last cluster resets both words for the next launch, which reads them only
+// after this grid has completed.
 __device__ __forceinline__ void work_done(int* work, int n_clusters) {
   __threadfence();
   if (atomicAdd(work + 1, 1) == n_clusters - 1) {
@@ -602,6 +603,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       }
       st_cluster_u32(rec + 4u * (3 * L::kRings), static_cast<uint32_t>(n_q[0]));
       st_cluster_u32(rec + 4u * (3 * L::kRings + 1), static_cast<uint32_t>(n_q[1]));
+      // this cluster takes no more items
+      if (dyn && leader) tc2::work_done(args.work, n_clusters);
     }
     __syncwarp();
   } else if (warp == Cfg::kMmaWarp) {
@@ -1187,13 +1190,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
 
   tc_fence_before();
   __syncthreads();
-  // the pair's MMAs and TMEM reads are over in both CTAs, and both producers'
-  // load records are in the leader's shared memory
+  if (threadIdx.x == 0) st_cluster_u32(mapa_shared(base + L::kPeerAbort, rank ^ 1u), static_cast<uint32_t>(*abort_flag));
+  // the pair's MMAs and TMEM reads are over in both CTAs, both producers' load
+  // records are in the leader's shared memory, and each CTA knows whether the
+  // other one gave up
   cluster_sync();
   if (warp == Cfg::kMmaWarp) {
     tc_fence_after();
     tmem_dealloc_pair(tmem, kTmemCols);
   }
+  // Every load has landed when neither CTA gave up: each was waited for before
+  // the MMAs that read it.  (Settling them all the same, with a second barrier
+  // behind, and resetting the work counter after it took 1 us of the 3 us
+  // between the last MMA and the exit.)
+  if (*abort_flag == 0 && *reinterpret_cast<const volatile int*>(base_ptr + L::kPeerAbort) == 0) return;
   if (leader && warp == Cfg::kProducerWarp && lane == 0) {
     // Every K, V and Q load of either CTA must land before that CTA exits.
     // The leader arms a phase for both halves before it issues its own, and
@@ -1225,7 +1235,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   }
   // the follower leaves only once the leader has seen every load of the pair land
   cluster_sync();
-  if (dyn && leader && threadIdx.x == 0) tc2::work_done(args.work, n_clusters);
 }
 
 }  // namespace rc
