@@ -62,6 +62,7 @@ struct AttnArgs {
   // order by whichever cluster is free, and the last cluster to finish resets
   // both words
   int* work;
+  int32_t static_list;  // the work list was complete before this launch was made (a cache's, not one copied on the stream)
 };
 
 // One item whose key range was split into parts: the combine kernel merges

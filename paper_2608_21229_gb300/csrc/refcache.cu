@@ -282,6 +282,7 @@ struct Operands {
   void* o;
   float* lse;
   int* status = nullptr;  // the cache's own error word, if the launch is for a cache
+  bool static_list = false;  // the work list is a cache's (AttnArgs::static_list)
   int* work = nullptr;    // work counter of the CTA-pair kernel (two ints, zero between launches), or null
 };
 
@@ -358,6 +359,7 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
   a.timeout_ns = g_timeout_ns.load();
   a.status = op.status;
   a.work = op.work;
+  a.static_list = op.static_list ? 1 : 0;
   a.q = static_cast<const __nv_bfloat16*>(op.q);
   a.ka = static_cast<const __nv_bfloat16*>(op.ka);
   a.va = static_cast<const __nv_bfloat16*>(op.va);
@@ -966,7 +968,7 @@ int refcache_build(refcache_t* h, int layer, const void* q_static, const void* k
     cj.rows = h->cache_rows;
   }
   Operands op{q_static, h->static_rows, k_static, v_static, h->static_rows, nullptr, nullptr, 0, o_static, lse_static,
-              h->d_status, h->d_work};
+              h->d_status, true, h->d_work};
   rc = run_attention(h->d_build, h->n_build, h->H, h->D, op, softmax_scale, info, s,
                      h->build_items.items ? &h->build_items : nullptr, nullptr, h->n_copy > 0 ? &cj : nullptr);
   if (rc) return rc;
@@ -1002,7 +1004,7 @@ int refcache_build_in_slot(refcache_t* h, int layer, const void* q_static, const
               range_b ? h->cache_rows : 0,
               o_static,
               lse_static,
-              h->d_status, h->d_work};
+              h->d_status, true, h->d_work};
   rc = run_attention(h->d_build_slot, h->n_build_slot, h->H, h->D, op, softmax_scale, info,
                      static_cast<cudaStream_t>(stream));
   if (rc) return rc;
@@ -1031,7 +1033,7 @@ int step_attention(refcache_t* h, int layer, const void* q_live, const void* k_l
     refcache_kv_ptr(h, layer, &kslot, &vslot, nullptr);
   }
   Operands op{q_live, h->live_rows, k_live, v_live, h->live_rows, kslot, vslot, h->cache_rows, o_live, lse_live,
-              h->d_status, h->d_work};
+              h->d_status, true, h->d_work};
   return run_attention(h->d_step, h->n_step, h->H, h->D, op, softmax_scale, info, static_cast<cudaStream_t>(stream),
                        h->step_items.items ? &h->step_items : nullptr, use_f8 ? &f8 : nullptr);
 }
@@ -1082,7 +1084,7 @@ int full_attention(int batch, int num_heads, int head_dim, const int32_t* cu_seq
     cudaError_t e = cudaMemcpyAsync(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(work list)");
   }
-  Operands op{q, rows, k, v, rows, nullptr, nullptr, 0, o, lse, nullptr, work};
+  Operands op{q, rows, k, v, rows, nullptr, nullptr, 0, o, lse, nullptr, false, work};
   return run_attention(d_tasks, static_cast<int>(tasks.size()), num_heads, head_dim, op, softmax_scale, info, s);
 }
 
