@@ -170,9 +170,9 @@ REFCACHE_API size_t refcache_bytes(int num_layers, int mask_mode, const refcache
  * arithmetic does not.  full_attention does the same with a counter kept
  * beside its work list; full_attention_noalloc takes items in a fixed order
  * (the same results, bit for bit).  When the step's
- * items do not fill the last round of the GPU's CTA pairs evenly, the items of
- * that round are split by key range into 2-8 parts whose outputs a combine
- * kernel merges.  These lists and an fp32 workspace for the parts (parts x 256
+ * items do not fill the last round of the GPU's CTA pairs evenly and it ends the
+ * step sooner, the items of that round are split by key range into 2-8 parts whose
+ * outputs a combine kernel merges.  These lists and an fp32 workspace for the parts (parts x 256
  * rows x (head_dim + 1) x 4 bytes, e.g. 27 MB at 1024^2 with five references)
  * are one more cudaMalloc, freed by refcache_destroy.  Which step items are split depends on the whole
  * batch and the device, so a step output's last bits may differ between

@@ -432,26 +432,62 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
   return REFCACHE_OK;
 }
 
+// When a list of items, taken longest first by whichever of `clusters` CTA pairs
+// is free, is done (in key-tile times): `costs` is sorted here.
+double list_end(std::vector<double>& costs, int clusters) {
+  std::sort(costs.begin(), costs.end(), std::greater<double>());
+  std::vector<double> heap(static_cast<size_t>(clusters), 0.0);  // a min-heap of the pairs' end times
+  for (double c : costs) {
+    std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
+    heap.back() += c;
+    std::push_heap(heap.begin(), heap.end(), std::greater<double>());
+  }
+  return *std::max_element(heap.begin(), heap.end());
+}
+
 // Per-item list of `tasks` x heads (head-major, as the kernels enumerate
 // items) for `clusters` CTA pairs.  When the items do not fill the last round
-// of the persistent grid, the items of that round are split by key tiles into
-// s parts each (s chosen so that the parts fill the clusters best), which run
-// after the whole items; their results are merged by combine jobs.
-void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, std::vector<Task>* items,
+// of the persistent grid, the items of that round may be split by key tiles into
+// s parts each, which run after the whole items; their results are merged by
+// combine jobs.  Whether, and into how many, by the end of the list under these
+// costs, in key-tile times (0.8 us; measured on the kernel's timeline): an item's
+// start and epilogue 2 (E4M3: 6), a part's larger epilogue 1, and the combine
+// kernel 6 (its hand-overs with the attention kernels around it) plus 0.03 per
+// part.  (Splitting whenever the last round was not full cost the step with 1280
+// live and 2048 cached rows, 24 heads, 10 us in the combine and the parts to save
+// 6.)  Long lists, whose last round matters little, are not split.
+void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, bool f8, std::vector<Task>* items,
                 std::vector<CombineJob>* jobs, int* n_parts) {
   items->clear();
   jobs->clear();
   *n_parts = 0;
   const int64_t n = static_cast<int64_t>(tasks.size()) * H;
   if (n == 0 || clusters < 1) return;
+  constexpr double kPart = 1.0, kCombine = 6.0, kCombinePart = 0.03;
+  const double item_cost = f8 ? 6.0 : 2.0;
+  constexpr int64_t kLongList = 20000;
+  auto key_tiles = [&](const Task& t) { return (t.a_len + tile - 1) / tile + (t.b_len + tile - 1) / tile; };
   const int64_t rem = n % clusters;
   int best_s = 1;
-  double best = 1.0;  // item-times the last round costs
-  if (rem > 0) {
-    for (int cand : {2, 3, 4, 6, 8}) {
-      const double cost = static_cast<double>((rem * cand + clusters - 1) / clusters) / cand;
-      if (cost < best - 1e-9) {
-        best = cost;
+  if (rem > 0 && n <= kLongList) {
+    double best = 0.0;
+    for (int cand : {1, 2, 3, 4, 6, 8}) {
+      std::vector<double> costs;
+      int64_t parts = 0;
+      for (int64_t i = 0; i < n; ++i) {
+        const int nkv = key_tiles(tasks[static_cast<size_t>(i % static_cast<int64_t>(tasks.size()))]);
+        const int s_here = i < n - rem ? 1 : std::min(cand, nkv / 4);
+        if (s_here < 2) {
+          costs.push_back(nkv + item_cost);
+          continue;
+        }
+        parts += s_here;
+        for (int k = 0; k < s_here; ++k)
+          costs.push_back(static_cast<double>(nkv) * (k + 1) / s_here - static_cast<double>(nkv) * k / s_here + item_cost + kPart);
+      }
+      const double end = list_end(costs, clusters) + (parts > 0 ? kCombine + kCombinePart * static_cast<double>(parts) : 0.0);
+      if (cand == 1 || end < best - 1e-9) {
+        best = end;
         best_s = cand;
       }
     }
@@ -737,7 +773,7 @@ int plan_split_items(refcache* h, DeviceInfo* info, const std::vector<Task>& bt,
   std::vector<Task> si, bi;
   std::vector<CombineJob> sj;
   int parts = 0;
-  plan_items(st, h->H, clusters, tile, &si, &sj, &parts);
+  plan_items(st, h->H, clusters, tile, f8, &si, &sj, &parts);
   si = longest_first(std::move(si), tile);
   for (int hd = 0; hd < h->H; ++hd)
     for (Task t : bt) {
