@@ -59,7 +59,7 @@
  *     kernels (no allocation, no copy), so they can be captured in a CUDA graph and replayed, once a
  *     first call on the device has run outside the capture (the kernels'
  *     attributes are set on first use).  full_attention is not capturable
- *     (it copies its work list from host memory).
+ *     (it may copy its work list from host memory).
  */
 #ifndef REFCACHE_H
 #define REFCACHE_H

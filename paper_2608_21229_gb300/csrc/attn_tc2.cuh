@@ -278,7 +278,8 @@ template <bool kF8, int kBN, int kDG>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::kThreads, 1)
     attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ka,
                     const __grid_constant__ CUtensorMap tm_va, const __grid_constant__ CUtensorMap tm_kb,
-                    const __grid_constant__ CUtensorMap tm_vb, const AttnArgs args) {
+                    const __grid_constant__ CUtensorMap tm_vb, const AttnArgs args,
+                    const __grid_constant__ Spans spans) {
   using namespace tc;
   using tc2::kQTile;
   using Cfg = tc2::Cfg<kF8, kBN>;
@@ -407,6 +408,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     return wait_cl(full, parity, ctl, where) && (leader || mbar_try_wait_acquire_cluster(full, parity));
   };
   auto ring_done = [&](int k) { mbar_arrive_cluster(lbar(L::kItemEmpty + k % tc2::kItemSlots)); };
+  // item `it` of the work list
+  auto fetch_item = [&](int it, Task& t, int& head) {
+    if (spans.n == 0) {
+      decode_item(args, it, t, head);
+      return;
+    }
+    head = it / args.n_tasks;
+    const int task = it - head * args.n_tasks;
+    int i = 0;
+    while (i + 1 < spans.n && spans.span[i + 1].task0 <= task) ++i;
+    const int r = (task - spans.span[i].task0) * args.rows_per_task;
+    t = Task{spans.span[i].row0 + r, min(args.rows_per_task, spans.span[i].len - r), spans.span[i].row0, spans.span[i].len,
+             0, 0, head, 0};
+  };
   // the leader's producer (one lane): item k, whose head is -1 when none is left
   auto publish = [&](int k, const Task& t, int head, int q_buf) {
     const uint4 lo = make_uint4(t.q_row0, t.q_rows | q_buf << 16, t.a_row0, t.a_len);  // (Q buffer: for the epilogue)
@@ -426,7 +441,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   if (args.static_list && leader && warp == Cfg::kProducerWarp && lane == 0) {
     Task t;
     int head;
-    decode_item(args, cluster, t, head);
+    fetch_item(cluster, t, head);
     publish(0, t, head, 0);
     first_keys = t.a_len + t.b_len > 0;
   }
@@ -472,7 +487,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           pub_item = static_cast<int>(min(it, static_cast<int64_t>(args.n_items)));
         } else if (pub_step == 1) {
           if (pub_item < args.n_items)
-            decode_item(args, pub_item, pub_task, pub_head);
+            fetch_item(pub_item, pub_task, pub_head);
           else
             pub_head = -1;
         } else {

@@ -65,6 +65,17 @@ struct AttnArgs {
   int32_t static_list;  // the work list was complete before this launch was made (a cache's, not one copied on the stream)
 };
 
+// The work list of a full recompute of up to kMaxSpans requests as a kernel
+// parameter: request i is rows [row0, row0 + len), its tasks (256 rows each) are
+// numbers [task0, ...) and attend all of its rows.  n = 0: the list is in memory.
+constexpr int kMaxSpans = 32;
+struct Spans {
+  struct {
+    int32_t row0, len, task0;
+  } span[kMaxSpans];
+  int32_t n;
+};
+
 // One item whose key range was split into parts: the combine kernel merges
 // parts [part0, part0 + nparts) of the workspace into rows [q_row0, q_row0 +
 // q_rows) of `head`.

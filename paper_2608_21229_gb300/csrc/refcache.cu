@@ -232,7 +232,8 @@ int tc2_clusters(DeviceInfo* info, int* clusters_out) {
 
 // The CTA-pair kernel: grid = 2 x the clusters that fit at once.
 template <bool kF8, int kBN, int kDG>
-int launch_tc2(const CUtensorMap (&maps)[5], const AttnArgs& a, DeviceInfo* info, cudaStream_t s) {
+int launch_tc2(const CUtensorMap (&maps)[5], const AttnArgs& a, const rc::Spans& spans, DeviceInfo* info,
+               cudaStream_t s) {
   constexpr uint32_t smem = rc::tc2::SmemT<kF8, kBN>::kDynamic;
   int max_clusters = 0;
   int rc = tc2_clusters<kF8, kBN, kDG>(info, &max_clusters);
@@ -251,7 +252,8 @@ int launch_tc2(const CUtensorMap (&maps)[5], const AttnArgs& a, DeviceInfo* info
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaError_t e =
-      cudaLaunchKernelEx(&cfg, rc::attn_tc2_kernel<kF8, kBN, kDG>, maps[0], maps[1], maps[2], maps[3], maps[4], a);
+      cudaLaunchKernelEx(&cfg, rc::attn_tc2_kernel<kF8, kBN, kDG>, maps[0], maps[1], maps[2], maps[3], maps[4], a,
+                         spans);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "attn_tc2_kernel launch");
   return REFCACHE_OK;
@@ -282,7 +284,7 @@ struct Operands {
   void* o;
   float* lse;
   int* status = nullptr;  // the cache's own error word, if the launch is for a cache
-  bool static_list = false;  // the work list is a cache's (AttnArgs::static_list)
+  bool static_list = false;  // the work list is a cache's, or `spans` (AttnArgs::static_list)
   int* work = nullptr;    // work counter of the CTA-pair kernel (two ints, zero between launches), or null
 };
 
@@ -344,7 +346,7 @@ int launch_copy(const CopyJob& c, const DeviceInfo* info, cudaStream_t s, bool b
 // launched right after it; with the mma.sync kernel it goes first.
 int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands& op, float scale, DeviceInfo* info,
                   cudaStream_t s, const ItemList* il = nullptr, const Fp8B* f8 = nullptr,
-                  const CopyJob* copy = nullptr) {
+                  const CopyJob* copy = nullptr, const rc::Spans& spans = rc::Spans{}) {
   if (n_tasks == 0) return copy ? launch_copy(*copy, info, s, false) : REFCACHE_OK;
   AttnArgs a{};
   a.tasks = d_tasks;
@@ -402,11 +404,11 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
     a.part_lse = il->part_lse;
   }
   if (f8)
-    rc = launch_tc2<true, 128, 128>(maps, a, info, s);
+    rc = launch_tc2<true, 128, 128>(maps, a, spans, info, s);
   else if (D == 128)
-    rc = tile == 128 ? launch_tc2<false, 128, 128>(maps, a, info, s) : launch_tc2<false, 192, 128>(maps, a, info, s);
+    rc = tile == 128 ? launch_tc2<false, 128, 128>(maps, a, spans, info, s) : launch_tc2<false, 192, 128>(maps, a, spans, info, s);
   else
-    rc = tile == 128 ? launch_tc2<false, 128, 64>(maps, a, info, s) : launch_tc2<false, 192, 64>(maps, a, info, s);
+    rc = tile == 128 ? launch_tc2<false, 128, 64>(maps, a, spans, info, s) : launch_tc2<false, 192, 64>(maps, a, spans, info, s);
   if (rc) return rc;
   if (copy && (rc = launch_copy(*copy, info, s, true)) != 0) return rc;
   if (il && il->n_jobs > 0) {
@@ -1086,20 +1088,45 @@ int full_attention(int batch, int num_heads, int head_dim, const int32_t* cu_seq
   if ((rc = enter_device(nullptr, &info)) != 0) return rc;
   int dev = 0;
   cudaGetDevice(&dev);
-  std::vector<Task> tasks;
-  for (int b = 0; b < batch; ++b) {
-    const int s0 = cu_seqlens[b], n = cu_seqlens[b + 1] - s0;
-    add_rows(tasks, task_rows(head_dim), s0, n, s0, n, 0, 0);
+  const int tr = task_rows(head_dim);
+  // Up to kMaxSpans requests go as a kernel parameter, longest first, so that no
+  // list is copied on the stream: the copy and the full stop around it, where
+  // otherwise one call's prologue overlaps the tail of the one before, cost 8 us a
+  // call (5 heads, 1964 rows: 22.3 us; now 16.4).  (The mma.sync kernel reads a list.)
+  rc::Spans spans{};
+  int64_t n_span_tasks = 0;
+  if (g_kernel.load() != REFCACHE_KERNEL_MMA_SYNC && batch <= rc::kMaxSpans) {
+    std::vector<int> order;
+    for (int b = 0; b < batch; ++b)
+      if (cu_seqlens[b + 1] > cu_seqlens[b]) order.push_back(b);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
+      return cu_seqlens[x + 1] - cu_seqlens[x] > cu_seqlens[y + 1] - cu_seqlens[y];
+    });
+    for (int b : order) {
+      auto& sp = spans.span[spans.n++];
+      sp.row0 = cu_seqlens[b];
+      sp.len = cu_seqlens[b + 1] - cu_seqlens[b];
+      sp.task0 = static_cast<int32_t>(n_span_tasks);
+      n_span_tasks += (sp.len + tr - 1) / tr;
+    }
+    if (spans.n == 0) return REFCACHE_OK;
   }
-  order_tasks(tasks);
-  if (tasks.empty()) return REFCACHE_OK;
+  std::vector<Task> tasks;
+  if (spans.n == 0) {
+    for (int b = 0; b < batch; ++b) {
+      const int s0 = cu_seqlens[b], n = cu_seqlens[b + 1] - s0;
+      add_rows(tasks, tr, s0, n, s0, n, 0, 0);
+    }
+    order_tasks(tasks);
+    if (tasks.empty()) return REFCACHE_OK;
+  }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Task* d_tasks = nullptr;
   int* work = nullptr;
   {
     std::lock_guard<std::mutex> lk(g_full_mu);
     FullScratch& fs = g_full[dev];
-    if (fs.cap < tasks.size()) {
+    if (fs.cap < std::max<size_t>(tasks.size(), 1)) {
       if (fs.buf) {
         cudaError_t e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
@@ -1117,11 +1144,15 @@ int full_attention(int batch, int num_heads, int head_dim, const int32_t* cu_seq
     }
     d_tasks = fs.buf;
     work = fs.work;
-    cudaError_t e = cudaMemcpyAsync(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(work list)");
+    if (!tasks.empty()) {
+      cudaError_t e = cudaMemcpyAsync(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice, s);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpyAsync(work list)");
+    }
   }
-  Operands op{q, rows, k, v, rows, nullptr, nullptr, 0, o, lse, nullptr, false, work};
-  return run_attention(d_tasks, static_cast<int>(tasks.size()), num_heads, head_dim, op, softmax_scale, info, s);
+  Operands op{q, rows, k, v, rows, nullptr, nullptr, 0, o, lse, nullptr, spans.n > 0, work};
+  const int64_t n_tasks = spans.n > 0 ? n_span_tasks : static_cast<int64_t>(tasks.size());
+  return run_attention(d_tasks, static_cast<int>(n_tasks), num_heads, head_dim, op, softmax_scale, info, s, nullptr, nullptr,
+                       nullptr, spans);
 }
 
 int full_attention_noalloc(int batch, int num_heads, int head_dim, const int32_t* cu_seqlens, const void* q,

@@ -90,3 +90,21 @@ def test_short_items_in_static_order(head_dim):
         assert rcb.status() == rcb.OK, rcb.last_error()
         outs.append((o, lse))
     assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+
+
+@pytest.mark.parametrize("batch", [1, 31, 32, 33])
+def test_full_attention_lists(batch):
+    """Work lists that travel as a kernel parameter (up to 32 requests, empty ones not counted) and in memory:
+    the same bytes as full_attention_noalloc's, whose list is in memory."""
+    lens = [0 if i % 5 == 3 else 1 + (i * 97) % 700 for i in range(batch)] + [0, 0]
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    q, k, v = (torch.randn(cu[-1], 3, 128, device="cuda", generator=torch.Generator("cuda").manual_seed(s)).to(torch.bfloat16)
+               for s in (4, 5, 6))
+    outs = []
+    for call in (rcb.full_attention, rcb.full_attention, rcb.full_attention_noalloc):  # two in a row: the counter is reset
+        o, lse = torch.full_like(q, float("nan")), torch.full((cu[-1], 3), float("nan"), device="cuda")
+        call(cu, q, k, v, o, lse)
+        outs.append((o, lse))
+    assert rcb.status() == rcb.OK, rcb.last_error()
+    for o, lse in outs[:2]:
+        assert torch.equal(o, outs[2][0]) and torch.equal(lse, outs[2][1])
