@@ -227,26 +227,56 @@ __global__ void __launch_bounds__(128) attn_mma_kernel(const AttnArgs a) {
 }
 
 // Cache write (the copy of the static pass's R rows' K and V into the
-// persistent slot of one layer).  One block row per request segment.  It reads
-// only the static inputs, so it may run beside the prefill attention: launched
+// persistent slot of one layer).  A segment's rows are contiguous on both sides, so
+// the write is a list of pieces of 2 KB of K and of V (a segment's last may be
+// shorter); a warp takes every n-th, eight 16-byte units per lane in flight.
+// (Divided by segments, a short one's share of the blocks stood idle while the
+// longest one's copied on: build of five requests of 704 to 5030 rows, 23 heads
+// of 64, 357 us a call; now 328.)
+//
+// It reads only the static inputs, so it may run while the prefill ends: launched
 // as a programmatic dependent of that kernel it starts once the prefill's CTAs
-// are all running (and so the inputs' producers are complete), and it waits
-// for the prefill to complete before it exits, so that the work after it on
-// the stream sees both.
+// are all running (and so the inputs' producers are complete), its CTAs find room
+// as the prefill's leave, and it waits for the prefill to complete before it
+// exits, so that the work after it on the stream sees both.
 struct CopySeg {
-  int32_t src_row0, dst_row0, nrows, pad;
+  int32_t src_row0, dst_row0, nrows, piece0;  // piece0: the segment's first piece
 };
-__global__ void copy_rows_kernel(const CopySeg* segs, const uint4* __restrict__ src_k,
-                                 const uint4* __restrict__ src_v, uint4* __restrict__ dst_k,
-                                 uint4* __restrict__ dst_v, int row_u4) {
+constexpr int kCopyPiece = 2048;  // bytes, of K and of V
+constexpr int kCopyThreads = 256;
+struct CopyArgs {
+  const CopySeg* segs;
+  int32_t n_segs, n_pieces;
+  int64_t row_bytes;
+  const uint8_t *src_k, *src_v;
+  uint8_t *dst_k, *dst_v;
+};
+__global__ void __launch_bounds__(kCopyThreads) copy_rows_kernel(const CopyArgs c) {
   if (threadIdx.x == 0) grid_launch_dependents();
-  const CopySeg s = segs[blockIdx.y];
-  const int64_t n = static_cast<int64_t>(s.nrows) * row_u4;
-  const int64_t so = static_cast<int64_t>(s.src_row0) * row_u4, d0 = static_cast<int64_t>(s.dst_row0) * row_u4;
-  for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    dst_k[d0 + i] = src_k[so + i];
-    dst_v[d0 + i] = src_v[so + i];
+  constexpr int kDepth = kCopyPiece / 512;
+  const int lane = threadIdx.x & 31;
+  const int64_t n_warps = static_cast<int64_t>(gridDim.x) * (kCopyThreads / 32);
+  const int64_t w = static_cast<int64_t>(blockIdx.x) * (kCopyThreads / 32) + (threadIdx.x >> 5);
+  int seg = 0;
+  for (int64_t q = w; q < c.n_pieces; q += n_warps) {
+    while (seg + 1 < c.n_segs && q >= c.segs[seg + 1].piece0) ++seg;
+    const CopySeg s = c.segs[seg];
+    const int64_t off = (q - s.piece0) * kCopyPiece;
+    const int64_t so = s.src_row0 * c.row_bytes + off, d0 = s.dst_row0 * c.row_bytes + off;
+    const int n = static_cast<int>(min(static_cast<int64_t>(kCopyPiece), s.nrows * c.row_bytes - off) / 16) - lane;
+    uint4 k[kDepth], v[kDepth];
+#pragma unroll
+    for (int u = 0; u < kDepth; ++u)
+      if (32 * u < n) {
+        k[u] = reinterpret_cast<const uint4*>(c.src_k + so)[lane + 32 * u];
+        v[u] = reinterpret_cast<const uint4*>(c.src_v + so)[lane + 32 * u];
+      }
+#pragma unroll
+    for (int u = 0; u < kDepth; ++u)
+      if (32 * u < n) {
+        reinterpret_cast<uint4*>(c.dst_k + d0)[lane + 32 * u] = k[u];
+        reinterpret_cast<uint4*>(c.dst_v + d0)[lane + 32 * u] = v[u];
+      }
   }
   grid_dependency_wait();
 }

@@ -29,6 +29,7 @@
 
 using rc::AttnArgs;
 using rc::CombineJob;
+using rc::CopyArgs;
 using rc::CopySeg;
 using rc::QuantTile;
 using rc::Task;
@@ -308,35 +309,22 @@ struct ItemList {
   float* part_lse = nullptr;
 };
 
-// The build's cache write: copy_rows_kernel over the request segments.
-struct CopyJob {
-  const CopySeg* segs = nullptr;
-  int n_segs = 0;
-  const void *src_k = nullptr, *src_v = nullptr;
-  void *dst_k = nullptr, *dst_v = nullptr;
-  int row_u4 = 0;
-  int64_t rows = 0;
-};
-
-// `beside`: launched as a programmatic dependent of the kernel before it, so
-// that it runs next to that kernel (its grid is kept to two CTAs per SM, which
-// fit beside the attention kernel's CTAs).
-int launch_copy(const CopyJob& c, const DeviceInfo* info, cudaStream_t s, bool beside) {
-  const int64_t per_seg = beside ? std::max(1, 2 * info->num_sms / c.n_segs) : 1024;
-  dim3 grid(static_cast<unsigned>(std::min<int64_t>(per_seg, (c.rows * c.row_u4 + 255) / 256 / c.n_segs + 1)),
-            static_cast<unsigned>(c.n_segs));
+// The build's cache write.  `beside`: launched as a programmatic dependent of the
+// kernel before it.  Three CTAs per SM: with two or four a single request's copy
+// was 1-4 % of the build slower (64 + 2048 and 128 + 4096 rows), more for many
+// requests.
+int launch_copy(const CopyArgs& c, const DeviceInfo* info, cudaStream_t s, bool beside) {
+  constexpr int64_t kWarps = rc::kCopyThreads / 32;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(256, 1, 1);
+  cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>(3 * info->num_sms, (c.n_pieces + kWarps - 1) / kWarps)), 1, 1);
+  cfg.blockDim = dim3(rc::kCopyThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = beside ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, rc::copy_rows_kernel, c.segs, static_cast<const uint4*>(c.src_k),
-                                     static_cast<const uint4*>(c.src_v), static_cast<uint4*>(c.dst_k),
-                                     static_cast<uint4*>(c.dst_v), c.row_u4);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, rc::copy_rows_kernel, c);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "copy_rows_kernel launch");
   return REFCACHE_OK;
@@ -346,7 +334,7 @@ int launch_copy(const CopyJob& c, const DeviceInfo* info, cudaStream_t s, bool b
 // launched right after it; with the mma.sync kernel it goes first.
 int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands& op, float scale, DeviceInfo* info,
                   cudaStream_t s, const ItemList* il = nullptr, const Fp8B* f8 = nullptr,
-                  const CopyJob* copy = nullptr, const rc::Spans& spans = rc::Spans{}) {
+                  const CopyArgs* copy = nullptr, const rc::Spans& spans = rc::Spans{}) {
   if (n_tasks == 0) return copy ? launch_copy(*copy, info, s, false) : REFCACHE_OK;
   AttnArgs a{};
   a.tasks = d_tasks;
@@ -584,7 +572,7 @@ struct refcache {
   Task* d_step = nullptr;
   int n_step = 0;
   CopySeg* d_copy = nullptr;
-  int n_copy = 0;
+  int n_copy = 0, n_copy_pieces = 0;
   // per-item lists of the pair kernel, ordered for the persistent
   // grid (the step's with split items), in a separate allocation:
   // [build items | step items | step jobs | part_o | part_lse]
@@ -662,6 +650,7 @@ int cache_plan(int num_layers, int mode_flags, const refcache_segments_t* seg, r
   const int tr = task_rows(D);
   std::vector<Task> bt, st, bs;
   std::vector<CopySeg> cp;
+  int64_t n_pieces = 0;  // of the cache write
   int a0 = 0;  // first row of request b's anchors in the anchor tensors of refcache_build_in_slot
   for (int b = 0; b < B; ++b) {
     const int s0 = seg->cu_static[b], ns = seg->cu_static[b + 1] - s0, na = seg->n_anchor[b];
@@ -689,9 +678,12 @@ int cache_plan(int num_layers, int mode_flags, const refcache_segments_t* seg, r
       c.src_row0 = mode == REFCACHE_MASK_BEYOND_ALT ? s0 : s0 + na;
       c.dst_row0 = c0;
       c.nrows = nc;
+      c.piece0 = static_cast<int32_t>(n_pieces);
+      n_pieces += (static_cast<int64_t>(nc) * H * D * 2 + rc::kCopyPiece - 1) / rc::kCopyPiece;
       cp.push_back(c);
     }
   }
+  if (n_pieces > (1ll << 31) - 1) return fail(REFCACHE_ERR_INVALID_ARG, "cache rows too large");
   order_tasks(bt);
   order_tasks(st);
   order_tasks(bs);
@@ -728,6 +720,7 @@ int cache_plan(int num_layers, int mode_flags, const refcache_segments_t* seg, r
     h->anchor_rows = a0;
     h->n_step = static_cast<int>(st.size());
     h->n_copy = static_cast<int>(cp.size());
+    h->n_copy_pieces = static_cast<int>(n_pieces);
   }
   if (build_tasks) *build_tasks = std::move(bt);
   if (step_tasks) *step_tasks = std::move(st);
@@ -994,16 +987,16 @@ int refcache_build(refcache_t* h, int layer, const void* q_static, const void* k
   }
   void *kslot = nullptr, *vslot = nullptr;
   if (!h->f8) refcache_kv_ptr(h, layer, &kslot, &vslot, nullptr);
-  CopyJob cj;
+  CopyArgs cj{};
   if (h->n_copy > 0) {
     cj.segs = h->d_copy;
     cj.n_segs = h->n_copy;
-    cj.src_k = k_static;
-    cj.src_v = v_static;
-    cj.dst_k = kslot;
-    cj.dst_v = vslot;
-    cj.row_u4 = h->H * h->D * 2 / 16;
-    cj.rows = h->cache_rows;
+    cj.n_pieces = h->n_copy_pieces;
+    cj.row_bytes = static_cast<int64_t>(h->H) * h->D * 2;
+    cj.src_k = static_cast<const uint8_t*>(k_static);
+    cj.src_v = static_cast<const uint8_t*>(v_static);
+    cj.dst_k = static_cast<uint8_t*>(kslot);
+    cj.dst_v = static_cast<uint8_t*>(vslot);
   }
   Operands op{q_static, h->static_rows, k_static, v_static, h->static_rows, nullptr, nullptr, 0, o_static, lse_static,
               h->d_status, true, h->d_work};
