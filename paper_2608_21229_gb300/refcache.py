@@ -129,11 +129,19 @@ def _ptr(t) -> Optional[int]:
 
 
 def _stream(stream) -> Optional[int]:
-    import torch
-
     if stream is None:
-        stream = torch.cuda.current_stream()
+        global _raw_stream
+        if _raw_stream is None:
+            import torch
+
+            # the handle without a Stream object around it (3 us a call)
+            raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+            _raw_stream = (lambda: raw(device())) if raw else (lambda: torch.cuda.current_stream().cuda_stream)
+        return _raw_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+_raw_stream = None  # () -> the current stream's handle, once torch is in use
 
 
 def _check_thd(name, t, rows, H, D):
@@ -143,6 +151,29 @@ def _check_thd(name, t, rows, H, D):
         raise ValueError(f"{name} is required")
     if t.dtype != torch.bfloat16 or tuple(t.shape) != (rows, H, D):
         raise ValueError(f"{name}: expected bf16 [{rows}, {H}, {D}], got {t.dtype} {tuple(t.shape)}")
+
+
+_bf16 = None  # torch.bfloat16, once torch is in use
+
+
+def _thd_ptrs(named, rows, H, D):
+    """The device pointers of THD tensors, which _check_thd and _ptr check in
+    this order.  The first line is what a good call runs: the separate checks
+    took a third of the 11 us that the host spends on a small step."""
+    global _bf16
+    if _bf16 is None:
+        import torch
+
+        _bf16 = torch.bfloat16
+    shape = (rows, H, D)
+    for _, t in named:
+        if t is None or t.dtype is not _bf16 or t.shape != shape or not t.is_cuda or not t.is_contiguous():
+            break
+    else:
+        return [t.data_ptr() for _, t in named]
+    for name, t in named:
+        _check_thd(name, t, rows, H, D)
+    return [_ptr(t) for _, t in named]
 
 
 def set_kernel(name: str) -> str:
@@ -212,6 +243,8 @@ class RefCache:
     handed to refcache_create, so the library itself allocates nothing.
     """
 
+    _slots = None  # views of every layer's (K slot, V slot), laid out by the first kv()
+
     def __init__(self, seg: Segments, num_layers: int = 1, mask_mode: str = "beyond", device=None,
                  cache_dtype: str = "bf16"):
         import torch
@@ -246,6 +279,9 @@ class RefCache:
 
     def kv(self, layer: int):
         """(K slot, V slot) of a layer as bf16 [cache_rows, H, D] views of the cache memory."""
+        if self._slots is not None and self.h is not None and type(layer) is int and 0 <= layer < self.num_layers:
+            k, v = self._slots[layer]
+            return k[:], v[:]
         import torch
 
         k, v, rows = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_int64()
@@ -258,6 +294,13 @@ class RefCache:
             off = p.value - base
             return self.mem[off:off + n].view(torch.bfloat16).view(rows.value, H, D)
 
+        # the slots of all layers lie one after the other, K before V: views of them
+        # are laid out once, and a later call takes its layer's (asking the library for
+        # the addresses and viewing the bytes took 16 us a call)
+        first = k.value - base - 2 * n * layer
+        slots = self.mem[first:first + 2 * n * self.num_layers].view(torch.bfloat16).view(
+            self.num_layers, 2, rows.value, H, D)
+        self._slots = [(slots[i, 0], slots[i, 1]) for i in range(self.num_layers)]
         return view(k), view(v)
 
     def fp8(self, layer: int):
@@ -297,11 +340,9 @@ class RefCache:
 
     def build(self, layer, q, k, v, o, lse=None, scale=None, stream=None):
         H, D, n = self.seg.num_heads, self.seg.head_dim, self.seg.static_rows
-        for name, t in (("q", q), ("k", k), ("v", v), ("o", o)):
-            _check_thd(name, t, n, H, D)
+        ptrs = _thd_ptrs((("q", q), ("k", k), ("v", v), ("o", o)), n, H, D)
         scale = default_scale(D) if scale is None else scale
-        _check(load().refcache_build(self.h, layer, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), scale,
-                                     _stream(stream)))
+        _check(load().refcache_build(self.h, layer, *ptrs, _ptr(lse), scale, _stream(stream)))
 
     def build_in_slot(self, layer, q, k_anchor, v_anchor, o, lse=None, scale=None, stream=None):
         """The prefill of a layer whose cached rows' K/V the caller already
@@ -323,21 +364,17 @@ class RefCache:
 
     def step(self, layer, q, k, v, o, lse=None, scale=None, stream=None):
         H, D, n = self.seg.num_heads, self.seg.head_dim, self.seg.live_rows
-        for name, t in (("q", q), ("k", k), ("v", v), ("o", o)):
-            _check_thd(name, t, n, H, D)
+        ptrs = _thd_ptrs((("q", q), ("k", k), ("v", v), ("o", o)), n, H, D)
         scale = default_scale(D) if scale is None else scale
-        _check(load().step_attention(self.h, layer, _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse), scale,
-                                     _stream(stream)))
+        _check(load().step_attention(self.h, layer, *ptrs, _ptr(lse), scale, _stream(stream)))
 
 
 def full_attention(cu_seqlens, q, k, v, o, lse=None, scale=None, stream=None):
     rows, H, D = q.shape
     cu = list(cu_seqlens)
-    for name, t in (("q", q), ("k", k), ("v", v), ("o", o)):
-        _check_thd(name, t, cu[-1], H, D)
+    ptrs = _thd_ptrs((("q", q), ("k", k), ("v", v), ("o", o)), cu[-1], H, D)
     scale = default_scale(D) if scale is None else scale
-    _check(load().full_attention(len(cu) - 1, H, D, _arr(cu), _ptr(q), _ptr(k), _ptr(v), _ptr(o), _ptr(lse),
-                                 scale, _stream(stream)))
+    _check(load().full_attention(len(cu) - 1, H, D, _arr(cu), *ptrs, _ptr(lse), scale, _stream(stream)))
 
 
 def full_attention_noalloc(cu_seqlens, q, k, v, o, lse=None, scale=None, stream=None):
@@ -345,8 +382,6 @@ def full_attention_noalloc(cu_seqlens, q, k, v, o, lse=None, scale=None, stream=
     memory: the call allocates no device memory (see include/refcache.h)."""
     rows, H, D = q.shape
     cu = list(cu_seqlens)
-    for name, t in (("q", q), ("k", k), ("v", v), ("o", o)):
-        _check_thd(name, t, cu[-1], H, D)
+    ptrs = _thd_ptrs((("q", q), ("k", k), ("v", v), ("o", o)), cu[-1], H, D)
     scale = default_scale(D) if scale is None else scale
-    _check(load().full_attention_noalloc(len(cu) - 1, H, D, _arr(cu), _ptr(q), _ptr(k), _ptr(v), _ptr(o),
-                                         _ptr(lse), scale, _stream(stream)))
+    _check(load().full_attention_noalloc(len(cu) - 1, H, D, _arr(cu), *ptrs, _ptr(lse), scale, _stream(stream)))
