@@ -15,6 +15,7 @@
 #include <cstdio>
 #include <cstring>
 #include <functional>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -423,14 +424,22 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
 }
 
 // When a list of items, taken longest first by whichever of `clusters` CTA pairs
-// is free, is done (in key-tile times): `costs` is sorted here.
-double list_end(std::vector<double>& costs, int clusters) {
-  std::sort(costs.begin(), costs.end(), std::greater<double>());
+// is free, is done (in key-tile times).  `costs`: how many items of each cost.
+double list_end(const std::map<double, int64_t, std::greater<double>>& costs, int clusters) {
   std::vector<double> heap(static_cast<size_t>(clusters), 0.0);  // a min-heap of the pairs' end times
-  for (double c : costs) {
-    std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
-    heap.back() += c;
-    std::push_heap(heap.begin(), heap.end(), std::greater<double>());
+  for (const auto& [cost, n_items] : costs) {
+    int64_t n = n_items;
+    // while the pairs' ends lie within one item of each other, the next `clusters`
+    // equal items go one to each
+    if (n >= clusters && *std::max_element(heap.begin(), heap.end()) - heap.front() <= cost) {
+      for (double& e : heap) e += cost * static_cast<double>(n / clusters);
+      n %= clusters;
+    }
+    for (; n > 0; --n) {
+      std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
+      heap.back() += cost;
+      std::push_heap(heap.begin(), heap.end(), std::greater<double>());
+    }
   }
   return *std::max_element(heap.begin(), heap.end());
 }
@@ -445,7 +454,7 @@ double list_end(std::vector<double>& costs, int clusters) {
 // kernel 6 (its hand-overs with the attention kernels around it) plus 0.03 per
 // part.  (Splitting whenever the last round was not full cost the step with 1280
 // live and 2048 cached rows, 24 heads, 10 us in the combine and the parts to save
-// 6.)  Long lists, whose last round matters little, are not split.
+// 6.)
 void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, bool f8, std::vector<Task>* items,
                 std::vector<CombineJob>* jobs, int* n_parts) {
   items->clear();
@@ -455,25 +464,23 @@ void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, b
   if (n == 0 || clusters < 1) return;
   constexpr double kPart = 1.0, kCombine = 6.0, kCombinePart = 0.03;
   const double item_cost = f8 ? 6.0 : 2.0;
-  constexpr int64_t kLongList = 20000;
   auto key_tiles = [&](const Task& t) { return (t.a_len + tile - 1) / tile + (t.b_len + tile - 1) / tile; };
+  const int64_t n_tasks = static_cast<int64_t>(tasks.size());
   const int64_t rem = n % clusters;
   int best_s = 1;
-  if (rem > 0 && n <= kLongList) {
+  if (rem > 0) {
     double best = 0.0;
     for (int cand : {1, 2, 3, 4, 6, 8}) {
-      std::vector<double> costs;
+      std::map<double, int64_t, std::greater<double>> costs;
+      for (const Task& t : tasks) costs[key_tiles(t) + item_cost] += H;
       int64_t parts = 0;
-      for (int64_t i = 0; i < n; ++i) {
-        const int nkv = key_tiles(tasks[static_cast<size_t>(i % static_cast<int64_t>(tasks.size()))]);
-        const int s_here = i < n - rem ? 1 : std::min(cand, nkv / 4);
-        if (s_here < 2) {
-          costs.push_back(nkv + item_cost);
-          continue;
-        }
+      for (int64_t i = n - rem; i < n; ++i) {
+        const int nkv = key_tiles(tasks[static_cast<size_t>(i % n_tasks)]);
+        const int s_here = std::min(cand, nkv / 4);
+        if (s_here < 2) continue;
+        --costs[nkv + item_cost];
+        costs[static_cast<double>(nkv) / s_here + item_cost + kPart] += s_here;
         parts += s_here;
-        for (int k = 0; k < s_here; ++k)
-          costs.push_back(static_cast<double>(nkv) * (k + 1) / s_here - static_cast<double>(nkv) * k / s_here + item_cost + kPart);
       }
       const double end = list_end(costs, clusters) + (parts > 0 ? kCombine + kCombinePart * static_cast<double>(parts) : 0.0);
       if (cand == 1 || end < best - 1e-9) {
