@@ -42,78 +42,86 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 
 // grid (H, tiles, 2): blockIdx.z = 0 quantises the tile's K, 1 its V (heads
 // fastest, so that CTAs running together read neighbouring bytes of the same
-// rows); 256 threads.  Thread i takes rows [4 q, 4 q + 4) of the tile (q = i % 32) and
-// head-dim columns [16 p, 16 p + 16) (p = i / 32): per row one 32-byte run.
-// K codes go out row by row (16 bytes); V codes are transposed through shared
-// memory as one 32-bit word (four rows) per column, so the 32 threads of a
-// warp store 32 consecutive words.
+// rows); 256 threads.
+//
+// Bound by memory: 4 bytes read and 2 written per cached element of K and V.
+// Every warp instruction moves whole 128-byte lines: 16 lanes take one head of a
+// row (8 columns = 16 bytes each), so a load covers two rows, and thread
+// (row group g = i / 16, c = i % 16) holds rows [8 g, 8 g + 8), columns
+// [8 c, 8 c + 8).  K codes leave as they lie (8 bytes a lane).  V codes are
+// transposed 8 x 8 in registers and through shared memory: the 8-byte word of
+// rows [8 g, 8 g + 8) of column d is word g ^ ((d / 8) % 16) of the column's 128
+// bytes, which spreads both the stores (16 columns 8 apart) and the reads (a
+// column's 128 bytes) over all banks.  (With a lane per four rows each load and K
+// store touched 32 rows' sectors: build of a 1024^2 request with two references
+// 541 us, 42 of them here; now 525.)
 __global__ void __launch_bounds__(256, 3) quantize_cache_kernel(const QuantTile* __restrict__ tiles,
                                                                 const uint4* __restrict__ k, const uint4* __restrict__ v,
                                                                 uint8_t* __restrict__ k8, uint8_t* __restrict__ vt8,
                                                                 float4* __restrict__ scales, int H, int64_t rows_pad) {
   constexpr int D = 128;
   __shared__ float red[8];
-  __shared__ __align__(16) uint32_t vt[D][32 + 4];  // V^T codes of the tile: [d][row / 4], 4 rows per word
+  __shared__ __align__(16) uint2 vt[D][16];  // V^T codes of the tile: [d][word of 8 rows, swizzled]
   const QuantTile t = tiles[blockIdx.y];
   const int h = blockIdx.x;
   const bool is_v = blockIdx.z != 0;
-  const int q = threadIdx.x & 31;   // rows 4 q .. 4 q + 3
-  const int p = threadIdx.x >> 5;   // columns 16 p .. 16 p + 15
+  const int g = threadIdx.x >> 4;  // rows 8 g .. 8 g + 7
+  const int c = threadIdx.x & 15;  // columns 8 c .. 8 c + 7
   const int64_t row_u4 = static_cast<int64_t>(H) * D / 8;
-  const uint4* src = is_v ? v : k;
-  uint4 x[4][2];
+  const uint4* src = (is_v ? v : k) + static_cast<int64_t>(t.src_row0 + 8 * g) * row_u4 + h * (D / 8) + c;
+  uint4 x[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) x[r] = 8 * g + r < t.valid ? src[r * row_u4] : make_uint4(0, 0, 0, 0);
   float a = 0.f;
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int row = 4 * q + r;
+  for (int r = 0; r < 8; ++r) {
+    const uint32_t w[4] = {x[r].x, x[r].y, x[r].z, x[r].w};
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      x[r][c] = row < t.valid ? src[static_cast<int64_t>(t.src_row0 + row) * row_u4 + h * (D / 8) + 2 * p + c]
-                              : make_uint4(0, 0, 0, 0);
-      const uint32_t w[4] = {x[r][c].x, x[r][c].y, x[r][c].z, x[r][c].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) a = fmax3(a, fabsf(bf16_lo(w[e])), fabsf(bf16_hi(w[e])));
-    }
+    for (int e = 0; e < 4; ++e) a = fmax3(a, fabsf(bf16_lo(w[e])), fabsf(bf16_hi(w[e])));
   }
   const float amax = block_amax_256(a, red);
   const float inv = amax > 0.f ? __fdiv_rn(448.f, amax) : 0.f;
-  // codes of the 16 columns of row r: four words of four codes
-  uint32_t cw[4][4];
+  // codes of the 8 columns of row r: two words of four codes
+  uint2 cw[8];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const uint4& y = x[r][c];
-      cw[r][2 * c] = pack_e4m3x4(__fmul_rn(bf16_lo(y.x), inv), __fmul_rn(bf16_hi(y.x), inv),
-                                 __fmul_rn(bf16_lo(y.y), inv), __fmul_rn(bf16_hi(y.y), inv));
-      cw[r][2 * c + 1] = pack_e4m3x4(__fmul_rn(bf16_lo(y.z), inv), __fmul_rn(bf16_hi(y.z), inv),
-                                     __fmul_rn(bf16_lo(y.w), inv), __fmul_rn(bf16_hi(y.w), inv));
-    }
+  for (int r = 0; r < 8; ++r)
+    cw[r] = make_uint2(pack_e4m3x4(__fmul_rn(bf16_lo(x[r].x), inv), __fmul_rn(bf16_hi(x[r].x), inv),
+                                   __fmul_rn(bf16_lo(x[r].y), inv), __fmul_rn(bf16_hi(x[r].y), inv)),
+                       pack_e4m3x4(__fmul_rn(bf16_lo(x[r].z), inv), __fmul_rn(bf16_hi(x[r].z), inv),
+                                   __fmul_rn(bf16_lo(x[r].w), inv), __fmul_rn(bf16_hi(x[r].w), inv)));
   if (!is_v) {
-    uint8_t* krow = k8 + static_cast<int64_t>(t.dst_row0) * H * D + static_cast<int64_t>(h) * D + 16 * p;
+    const int64_t row = static_cast<int64_t>(H) * D;
+    uint8_t* dst = k8 + (t.dst_row0 + 8 * g) * row + static_cast<int64_t>(h) * D + 8 * c;
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
-      *reinterpret_cast<uint4*>(krow + static_cast<int64_t>(4 * q + r) * H * D) =
-          make_uint4(cw[r][0], cw[r][1], cw[r][2], cw[r][3]);
+    for (int r = 0; r < 8; ++r) *reinterpret_cast<uint2*>(dst + r * row) = cw[r];
     if (threadIdx.x == 0) scales[static_cast<int64_t>(t.dst_row0 >> 7) * H + h].x = __fdiv_rn(amax, 448.f);
     return;
   }
-  // column 16 p + 4 w + e: byte e of word w of each of the four rows
+  // column 8 c + 4 w + e: byte e of word w of each of the eight rows
 #pragma unroll
-  for (int w = 0; w < 4; ++w)
+  for (int w = 0; w < 2; ++w)
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      vt[16 * p + 4 * w + e][q] = __byte_perm(__byte_perm(cw[0][w], cw[1][w], 0x0040 + e * 0x0011),
-                                              __byte_perm(cw[2][w], cw[3][w], 0x0040 + e * 0x0011), 0x5410);
+    for (int e = 0; e < 4; ++e) {
+      uint32_t col[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const uint32_t r0 = w ? cw[4 * u].y : cw[4 * u].x, r1 = w ? cw[4 * u + 1].y : cw[4 * u + 1].x;
+        const uint32_t r2 = w ? cw[4 * u + 2].y : cw[4 * u + 2].x, r3 = w ? cw[4 * u + 3].y : cw[4 * u + 3].x;
+        col[u] = __byte_perm(__byte_perm(r0, r1, 0x0040 + e * 0x0011), __byte_perm(r2, r3, 0x0040 + e * 0x0011), 0x5410);
+      }
+      vt[8 * c + 4 * w + e][g ^ c] = make_uint2(col[0], col[1]);
+    }
   __syncthreads();
-  // V^T rows: 128 d rows of 128 codes, 16 bytes per thread and step
+  // V^T rows: 128 d rows of 128 codes, 16 bytes per thread and step: words
+  // 2 ch and 2 ch + 1 of row d lie side by side, exchanged where d / 8 is odd
   uint8_t* vbase = vt8 + static_cast<int64_t>(h) * D * rows_pad + t.dst_row0;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int idx = threadIdx.x + 256 * i;  // 0..1023 = d * 8 + chunk
-    const int d = idx >> 3, ch = idx & 7;
+    const int d = idx >> 3, ch = idx & 7, z = d >> 3;
+    const uint4 y = *reinterpret_cast<const uint4*>(&vt[d][2 * (ch ^ (z >> 1))]);
     *reinterpret_cast<uint4*>(vbase + static_cast<int64_t>(d) * rows_pad + 16 * ch) =
-        *reinterpret_cast<const uint4*>(&vt[d][4 * ch]);
+        z & 1 ? make_uint4(y.z, y.w, y.x, y.y) : y;
   }
   if (threadIdx.x == 0) {
     const float sv = __fdiv_rn(amax, 448.f);

@@ -108,3 +108,21 @@ def test_full_attention_lists(batch):
     assert rcb.status() == rcb.OK, rcb.last_error()
     for o, lse in outs[:2]:
         assert torch.equal(o, outs[2][0]) and torch.equal(lse, outs[2][1])
+
+
+#: cached rows of a request at the edges of the cache write's groups of eight rows
+#: and of its 128-row tiles
+ROWS = (1, 7, 8, 9, 63, 64, 65, 120, 121, 127, 128, 129, 249, 256)
+
+
+@pytest.mark.parametrize("heads", [1, 5])
+@pytest.mark.parametrize("mode", ["beyond", "beyond_alt"])
+def test_e4m3_cache_write_at_the_edges_of_row_groups(mode, heads):
+    reqs = tuple(workloads.Request(i % 2, 0, 1, n) for i, n in enumerate(ROWS))
+    w = workloads.Workload("quant_edges", heads, 128, reqs, 35)
+    static = list(workloads.static_qkv(w))
+    for i, t in enumerate(static[1:]):  # columns of one head at other scales, one tile of zeros
+        t[:, 0, 8 * i:8 * i + 3] *= 300.0
+        t[w.cu_static[3]:w.cu_static[4]] = 0
+    rcb.set_kernel("tcgen05")
+    fp8.check_cache(fp8.Fp8Run(w, mode=mode, static=tuple(static)), np.arange(heads))
