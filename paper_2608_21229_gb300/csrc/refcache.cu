@@ -32,6 +32,7 @@ using rc::AttnArgs;
 using rc::CombineJob;
 using rc::CopyArgs;
 using rc::CopySeg;
+using rc::QuantArgs;
 using rc::QuantTile;
 using rc::Task;
 
@@ -310,33 +311,41 @@ struct ItemList {
   float* part_lse = nullptr;
 };
 
-// The build's cache write.  `beside`: launched as a programmatic dependent of the
-// kernel before it.  Three CTAs per SM: with two or four a single request's copy
-// was 1-4 % of the build slower (64 + 2048 and 128 + 4096 rows), more for many
-// requests.
-int launch_copy(const CopyArgs& c, const DeviceInfo* info, cudaStream_t s, bool beside) {
+// The build's cache write: rows copied, or quantised into an E4M3 cache.
+struct CacheWrite {
+  CopyArgs copy{};    // n_pieces > 0: copied
+  QuantArgs quant{};  // n_tiles > 0: quantised
+};
+
+// `beside`: launched as a programmatic dependent of the kernel before it.  Three
+// copying CTAs per SM: with two or four a single request's copy was 1-4 % of the
+// build slower (64 + 2048 and 128 + 4096 rows), more for many requests.
+int launch_cache_write(const CacheWrite& w, const DeviceInfo* info, cudaStream_t s, bool beside) {
   constexpr int64_t kWarps = rc::kCopyThreads / 32;
+  const bool quant = w.quant.n_tiles > 0;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>(3 * info->num_sms, (c.n_pieces + kWarps - 1) / kWarps)), 1, 1);
-  cfg.blockDim = dim3(rc::kCopyThreads, 1, 1);
+  cfg.gridDim = quant ? dim3(static_cast<unsigned>(w.quant.num_heads), static_cast<unsigned>(w.quant.n_tiles), 2)
+                      : dim3(static_cast<unsigned>(std::min<int64_t>(3 * info->num_sms, (w.copy.n_pieces + kWarps - 1) / kWarps)));
+  cfg.blockDim = dim3(quant ? rc::kQuantThreads : rc::kCopyThreads, 1, 1);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = beside ? 1 : 0;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, rc::copy_rows_kernel, c);
+  cudaError_t e = quant ? cudaLaunchKernelEx(&cfg, rc::quantize_cache_kernel, w.quant)
+                        : cudaLaunchKernelEx(&cfg, rc::copy_rows_kernel, w.copy);
   if (e == cudaSuccess) e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, "copy_rows_kernel launch");
+  if (e != cudaSuccess) return cuda_fail(e, quant ? "quantize_cache_kernel launch" : "copy_rows_kernel launch");
   return REFCACHE_OK;
 }
 
-// `copy` (the build's cache write, if any) runs beside the pair kernel,
+// `write` (the build's cache write, if any) runs beside the pair kernel,
 // launched right after it; with the mma.sync kernel it goes first.
 int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands& op, float scale, DeviceInfo* info,
                   cudaStream_t s, const ItemList* il = nullptr, const Fp8B* f8 = nullptr,
-                  const CopyArgs* copy = nullptr, const rc::Spans& spans = rc::Spans{}) {
-  if (n_tasks == 0) return copy ? launch_copy(*copy, info, s, false) : REFCACHE_OK;
+                  const CacheWrite* write = nullptr, const rc::Spans& spans = rc::Spans{}) {
+  if (n_tasks == 0) return write ? launch_cache_write(*write, info, s, false) : REFCACHE_OK;
   AttnArgs a{};
   a.tasks = d_tasks;
   a.n_tasks = n_tasks;
@@ -359,7 +368,7 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
   if (static_cast<int64_t>(n_tasks) * H > (1ll << 30)) return fail(REFCACHE_ERR_INVALID_ARG, "too many work items");
   if (g_kernel.load() == REFCACHE_KERNEL_MMA_SYNC) {
     if (f8) return fail(REFCACHE_ERR_UNSUPPORTED, "the E4M3 cache runs on the tcgen05 kernel only");
-    int rc = copy ? launch_copy(*copy, info, s, false) : REFCACHE_OK;
+    int rc = write ? launch_cache_write(*write, info, s, false) : REFCACHE_OK;
     if (rc) return rc;
     return D == 64 ? launch_mma<64>(a, info, s) : launch_mma<128>(a, info, s);
   }
@@ -399,7 +408,7 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
   else
     rc = tile == 128 ? launch_tc2<false, 128, 64>(maps, a, spans, info, s) : launch_tc2<false, 192, 64>(maps, a, spans, info, s);
   if (rc) return rc;
-  if (copy && (rc = launch_copy(*copy, info, s, true)) != 0) return rc;
+  if (write && (rc = launch_cache_write(*write, info, s, true)) != 0) return rc;
   if (il && il->n_jobs > 0) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(static_cast<unsigned>((a.rows_per_task + rc::kCombineRows - 1) / rc::kCombineRows),
@@ -983,32 +992,35 @@ int refcache_build(refcache_t* h, int layer, const void* q_static, const void* k
   DeviceInfo* info = nullptr;
   if ((rc = enter_device(h, &info)) != 0) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (h->f8 && h->n_qtiles > 0) {
+  CacheWrite w;
+  if (h->n_qtiles > 0) {
     void *k8 = nullptr, *vt8 = nullptr, *sc = nullptr;
     refcache_fp8_ptr(h, layer, &k8, &vt8, &sc, nullptr);
-    rc::quantize_cache_kernel<<<dim3(static_cast<unsigned>(h->H), static_cast<unsigned>(h->n_qtiles), 2), 256, 0, s>>>(
-        h->d_qtiles, static_cast<const uint4*>(k_static), static_cast<const uint4*>(v_static),
-        static_cast<uint8_t*>(k8), static_cast<uint8_t*>(vt8), static_cast<float4*>(sc), h->H, h->rows_pad);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "quantize_cache_kernel launch");
-  }
-  void *kslot = nullptr, *vslot = nullptr;
-  if (!h->f8) refcache_kv_ptr(h, layer, &kslot, &vslot, nullptr);
-  CopyArgs cj{};
-  if (h->n_copy > 0) {
-    cj.segs = h->d_copy;
-    cj.n_segs = h->n_copy;
-    cj.n_pieces = h->n_copy_pieces;
-    cj.row_bytes = static_cast<int64_t>(h->H) * h->D * 2;
-    cj.src_k = static_cast<const uint8_t*>(k_static);
-    cj.src_v = static_cast<const uint8_t*>(v_static);
-    cj.dst_k = static_cast<uint8_t*>(kslot);
-    cj.dst_v = static_cast<uint8_t*>(vslot);
+    w.quant.tiles = h->d_qtiles;
+    w.quant.n_tiles = h->n_qtiles;
+    w.quant.num_heads = h->H;
+    w.quant.src_k = static_cast<const uint4*>(k_static);
+    w.quant.src_v = static_cast<const uint4*>(v_static);
+    w.quant.k8 = static_cast<uint8_t*>(k8);
+    w.quant.vt8 = static_cast<uint8_t*>(vt8);
+    w.quant.scales = static_cast<float4*>(sc);
+    w.quant.rows_pad = h->rows_pad;
+  } else if (h->n_copy > 0) {
+    void *kslot = nullptr, *vslot = nullptr;
+    refcache_kv_ptr(h, layer, &kslot, &vslot, nullptr);
+    w.copy.segs = h->d_copy;
+    w.copy.n_segs = h->n_copy;
+    w.copy.n_pieces = h->n_copy_pieces;
+    w.copy.row_bytes = static_cast<int64_t>(h->H) * h->D * 2;
+    w.copy.src_k = static_cast<const uint8_t*>(k_static);
+    w.copy.src_v = static_cast<const uint8_t*>(v_static);
+    w.copy.dst_k = static_cast<uint8_t*>(kslot);
+    w.copy.dst_v = static_cast<uint8_t*>(vslot);
   }
   Operands op{q_static, h->static_rows, k_static, v_static, h->static_rows, nullptr, nullptr, 0, o_static, lse_static,
               h->d_status, true, h->d_work};
   rc = run_attention(h->d_build, h->n_build, h->H, h->D, op, softmax_scale, info, s,
-                     h->build_items.items ? &h->build_items : nullptr, nullptr, h->n_copy > 0 ? &cj : nullptr);
+                     h->build_items.items ? &h->build_items : nullptr, nullptr, h->n_qtiles > 0 || h->n_copy > 0 ? &w : nullptr);
   if (rc) return rc;
   h->built[layer] = 1;
   return REFCACHE_OK;
