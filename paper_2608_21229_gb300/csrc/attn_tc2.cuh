@@ -30,7 +30,7 @@
 //   warp 4     TMA producer: this CTA's Q rows and its halves of the K and V
 //              tiles; completion is counted on the leader's barriers
 //   warp 5     both CTAs: TMEM allocation (a pair operation); leader only:
-//              the MMA warp (lane 0 issues every MMA and commit)
+//              the MMA warp (one elected lane issues every MMA and commit)
 //   warp 6     leader only: the gate warp, which does every mbarrier wait
 //              the MMAs depend on and hands each group to the MMA warp
 //              through a named barrier
@@ -63,7 +63,8 @@
 // in every role one after the other took about 5000 cycles per item, and the
 // epilogue's uncoalesced stores 2000.  MMA-thread waits around an item's start
 // went from 5100 to 2700 cycles; step with 1280 live and 2048 cached rows
-// (items of 9 tiles), 24 heads: 62.7 -> 60.7 us.
+// (items of 9 tiles), 24 heads: 62.7 -> 60.7 us (its last round was still split then;
+// now 43 us).
 //
 // Synchronisation is built so that the MMA thread waits on nothing itself: all
 // mbarrier waits are done by the gate warp: per group, the gate warp waits for
@@ -146,7 +147,7 @@ constexpr uint32_t kQTile = 128 * 128 * 2;
 // 12 P.V MMAs and 8 S MMAs of N = 192 (1536 tensor cycles per handshake
 // instead of 1024), and since the S MMAs that reuse a buffer overwrite the P
 // that the group's P.V MMAs read, a group issues all its P.V MMAs first.
-// With 128-key tiles P has buffers of its own and the two kinds interleave.
+// With 128-key tiles P has buffers of its own (the groups keep that order).
 template <bool kF8, int kBN>
 struct Cfg {
   static_assert(kBN == 128 || (kBN == 192 && !kF8), "key tiles of 128 keys, or 192 with the bf16 cache");
@@ -846,7 +847,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   } else {
     // ------------------------------------------------------------ softmax (both CTAs)
     // kH = 1: warp w (0-3) owns rows 32 w .. 32 w + 31 of this CTA's 128 rows
-    // (its TMEM lanes) and all 128 key columns.  kH = 2 (E4M3 kernel): warps w
+    // (its TMEM lanes) and all kBN key columns.  kH = 2 (E4M3 kernel): warps w
     // and w + 4 share those rows, warp w + 4 hh taking key columns and O
     // columns [64 hh, 64 hh + 64), so that two warps per SM sub-partition share
     // the exponentials.  Both read the whole S row, find the same row maximum

@@ -538,15 +538,12 @@ void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, b
 
 // Orders a per-item list for the CTA-pair kernel, which hands items out in
 // list order to whichever CTA pair is free (a work counter): longest items
-// first (MMA groups: key tiles + 2), items of equal length in their order
+// first (by key tiles), items of equal length in their order
 // (head-major, so that the pairs running at the same time share few heads'
 // K/V tiles in L2).  Only the order changes, not any item's arithmetic.
 std::vector<Task> longest_first(std::vector<Task> items, int tile) {
-  auto groups = [&](const Task& t) -> int64_t {
-    const int64_t nkv = (t.a_len + tile - 1) / tile + (t.b_len + tile - 1) / tile;
-    return nkv > 0 ? nkv + 2 : 0;
-  };
-  std::stable_sort(items.begin(), items.end(), [&](const Task& x, const Task& y) { return groups(x) > groups(y); });
+  auto key_tiles = [&](const Task& t) { return (t.a_len + tile - 1) / tile + (t.b_len + tile - 1) / tile; };
+  std::stable_sort(items.begin(), items.end(), [&](const Task& x, const Task& y) { return key_tiles(x) > key_tiles(y); });
   return items;
 }
 
