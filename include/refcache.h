@@ -114,9 +114,8 @@ extern "C" {
 #define REFCACHE_CACHE_FP8 0x100
 
 /* Kernel selection (refcache_set_kernel): the tcgen05/TMEM/TMA kernel is the
- * default (on CTA pairs with 192-key tiles for the bf16 cache; head_dim 64
- * runs on the same kernel with the head dim padded to 128 inside shared
- * memory); the mma.sync kernel is the recompiled legacy-tensor-core baseline;
+ * default (on CTA pairs with 192-key tiles for the bf16 cache, at both head
+ * dims); the mma.sync kernel is the recompiled legacy-tensor-core baseline;
  * TCGEN05_K128 is the same tcgen05 pair kernel with 128-key tiles, kept as a
  * comparison point (the E4M3 cache always uses 128-key tiles). */
 #define REFCACHE_KERNEL_TCGEN05 0

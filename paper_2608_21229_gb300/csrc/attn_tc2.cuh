@@ -2,8 +2,7 @@
 // (task, head) item, O = softmax(scale * Q K^T) V over the task's visible keys
 // (key ranges A then B; see common.cuh), scores, softmax and accumulation in
 // fp32 and P rounded to bf16 for P.V, with every MMA issued over two CTAs on
-// neighbouring SMs (tcgen05 cta_group::2, M = 256).  Head dim 128, or 64
-// padded to 128 inside shared memory (see the kernel's kDG).
+// neighbouring SMs (tcgen05 cta_group::2, M = 256).  Head dim 128 or 64.
 //
 // Why pairs: with one 128-row query tile per SM, each S/P.V pair of MMAs
 // (1024 tensor cycles at 128-key tiles) needs a fresh 32 KB K tile and 32 KB
@@ -12,8 +11,8 @@
 // memory delivers in 1024 cycles (128 bytes per cycle), so the tensor core
 // waits for data.  A CTA pair shares every K/V tile: CTA r holds keys
 // [kBN/2 r, kBN/2 (r + 1)) of each K tile and head-dim columns [64 r, 64 r +
-// 64) of each V tile (the B operand of a cta_group::2 MMA is split along N
-// between the two CTAs), while each CTA keeps its own 128 query rows (A is
+// 64) of each V tile (32 of 64 at head dim 64; the B operand of a cta_group::2
+// MMA is split along N between the two CTAs), while each CTA keeps its own 128 query rows (A is
 // split along M).  Per SM this halves the tile bytes fetched and the
 // B-operand bytes read, for the same MMA work.
 //
@@ -162,7 +161,7 @@ struct Cfg {
   static constexpr int kStages = kBN == 128 ? 4 : 3;     // K and V ring slots (shared memory: 2 Q + slots <= 227 KB)
   static constexpr uint32_t kKBox = (kBN / 2) * 128;     // one K box: kBN / 2 rows x 128 bytes
   static constexpr uint32_t kKHalf = 2 * kKBox;          // this CTA's kBN / 2 keys x 128 d of a K tile
-  static constexpr uint32_t kVHalf = kBN * 64 * 2;       // kBN keys x this CTA's 64 d of a V tile
+  static constexpr uint32_t kVHalf = kBN * 64 * 2;       // kBN keys x this CTA's 64 d of a V tile (head dim 64: 32)
   static constexpr uint32_t kStage = kKHalf + kVHalf;
   static constexpr bool kPOverS = kBN != 128;
   static constexpr uint32_t kColS = 0;                   // S buffer b at kColS + b * kBN
@@ -269,12 +268,14 @@ __device__ __forceinline__ void work_done(int* work, int n_clusters) {
 }
 }  // namespace tc2
 
-// kDG: the tensors' head dim.  At 64 the tiles keep the layout of head dim
-// 128 with the upper 64 columns as zero padding: Q and K tiles load only
-// their first 64-column box (S = Q K^T takes the first four K = 16 steps), the
-// second CTA of a pair holds the upper half of V's columns, which it never
-// loads but zeroes once (P V keeps N = 128; O's upper 64 columns stay zero and
-// are never read).
+// kDG: the head dim.  At 64 a Q or K row is one 64-column box (S = Q K^T takes
+// four K = 16 steps) and each CTA of a pair holds 32 of V's 64 columns: 64-byte
+// rows with the 64-byte swizzle, P V with N = 64, O in 64 columns of tensor
+// memory.  (Padded to 128 columns, with zeros for the second CTA's half, P V did
+// twice the work.  The softmax warps bound this head dim, but the MMAs lie on the
+// way from P to the next S: in-place build of three requests with 48 heads, 1614
+// to 6271 rows, 574 -> 544 us; step of 320 live and 256 cached rows, 4 heads,
+// 8.89 -> 8.72 us.)
 template <bool kF8, int kBN, int kDG>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::kThreads, 1)
     attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ka,
@@ -286,7 +287,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   using Cfg = tc2::Cfg<kF8, kBN>;
   constexpr uint32_t kKBox = Cfg::kKBox;
   constexpr uint32_t kKHalf = Cfg::kKHalf;
-  constexpr uint32_t kVHalf = Cfg::kVHalf;
+  constexpr uint32_t kVHalf = kBN * kDG;  // bytes of this CTA's V half: kBN keys x kDG / 2 columns
+  constexpr uint32_t kVStep = 16 * kDG;   // of which 16 keys
   constexpr uint32_t kStage = Cfg::kStage;
   constexpr int kStages = Cfg::kStages;
   constexpr uint32_t kColS = Cfg::kColS, kColP = Cfg::kColP, kPStride = Cfg::kPStride, kColO = Cfg::kColO;
@@ -298,14 +300,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   using tc2::kKHalf8;
   using tc2::kVHalf8;
   using L = tc2::SmemT<kF8, kBN>;
-  constexpr int D = tc2::kD;   // head-dim columns of the tiles (P V's N)
+  constexpr int D = tc2::kD;   // the larger head dim
   constexpr int DG = kDG;      // head dim of the tensors
-  static_assert(DG == D || (DG == 64 && !kF8), "head dim 128, or 64 (bf16 cache) padded to 128");
+  static_assert(DG == D || (DG == 64 && !kF8), "head dim 128, or 64 (bf16 cache)");
   constexpr int kQBoxes = DG / 64;  // 64-column boxes of a Q or K row loaded
   auto slot_of = [](int t) -> int { return tc2::slot_of<kStages>(t); };
   auto slot_parity = [](int t) -> uint32_t { return tc2::slot_parity<kStages>(t); };
   constexpr uint32_t kIdescS = idesc_bf16_f32(256, kBN, false);
-  constexpr uint32_t kIdescO = idesc_bf16_f32(256, D, true);
+  constexpr uint32_t kIdescO = idesc_bf16_f32(256, DG, true);
   constexpr uint32_t kIdesc8 = idesc_e4m3_f32(256, 128);  // S and O of cached tiles (N = 128 keys or d)
 
   extern __shared__ uint8_t smem_raw[];
@@ -362,16 +364,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     prefetch_tmap(&tm_va);
     prefetch_tmap(&tm_kb);
     prefetch_tmap(&tm_vb);
-  }
-  if constexpr (DG != D) {
-    // head dim 64: the second CTA's V half of every ring slot is the zero padding
-    // of the upper 64 head-dim columns (written once; that CTA never loads V)
-    if (rank == 1) {
-      constexpr uint32_t kChunks = kVHalf / 16;
-      for (uint32_t i = threadIdx.x; i < kStages * kChunks; i += blockDim.x)
-        st_shared_v4(base + L::kRing + (i / kChunks) * kStage + kKHalf + (i % kChunks) * 16u, make_uint4(0, 0, 0, 0));
-      fence_proxy_async_smem();
-    }
   }
   if (warp == Cfg::kMmaWarp) {
     tmem_alloc_pair(smem_u32(tmem_holder), kTmemCols);
@@ -537,20 +529,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           const int slot = slot_of(t);
           const TileSrc vs = tc2::tile_src<kBN>(vt, v_na, vj);
           const bool v8 = kF8 && vs.in_b;
-          const bool v_here = DG == D || rank == 0;  // at head dim 64 only the first CTA loads V
           const uint32_t vb = v8 ? kVHalf8 : kVHalf;
           const uint32_t dst = base + L::kRing + static_cast<uint32_t>(slot) * kStage + kKHalf;
           const uint32_t full = lbar(L::kVFull + slot);
-          if (leader) mbar_arrive_expect_tx(bar(L::kVFull + slot), (DG == D ? 2 : 1) * vb);
+          if (leader) mbar_arrive_expect_tx(bar(L::kVFull + slot), 2 * vb);
           ++n_ring[kStages + slot];
-          own_bytes[kStages + slot] = v_here ? vb : 0u;
-          other_bytes[kStages + slot] = DG == D || rank == 1 ? vb : 0u;
-          // E4M3: V^T rows d in [64 r, 64 r + 64), all 128 keys; bf16: head-dim
-          // columns [64 r, 64 r + 64) of all kBN keys
-          if (v_here) {
-            const int d0 = vt.head * DG + 64 * static_cast<int>(rank);
-            tma_load_2d_pair(dst, vs.in_b ? &tm_vb : &tm_va, full, v8 ? vs.row : d0, v8 ? d0 : vs.row);
-          }
+          own_bytes[kStages + slot] = vb;
+          other_bytes[kStages + slot] = vb;
+          // head-dim columns [DG/2 r, DG/2 (r + 1)) of all kBN keys (E4M3: these
+          // rows of V^T, all 128 keys)
+          const int d0 = vt.head * DG + DG / 2 * static_cast<int>(rank);
+          tma_load_2d_pair(dst, vs.in_b ? &tm_vb : &tm_va, full, v8 ? vs.row : d0, v8 ? d0 : vs.row);
           ++vj;
         }
         // the K side's next item, once its tiles are loaded; the leader chooses
@@ -641,7 +630,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     if (leader) {
       // descriptors of ring slot 0 (slot s: + s * kStage / 16) and of Q buffer 0
       const uint64_t kd0 = sdesc_sw128(base + L::kRing, 16, 1024);
-      const uint64_t vd0 = sdesc_sw128(base + L::kRing + kKHalf, Cfg::kVHalf, 1024);
+      const uint64_t vd0 = DG == 64 ? sdesc_sw64(base + L::kRing + kKHalf, kVHalf, 512)
+                                    : sdesc_sw128(base + L::kRing + kKHalf, kVHalf, 1024);
       const uint64_t qdesc0 = sdesc_sw128(base + L::kQ, 16, 1024);
       // E4M3 operands: Q8 (128 rows x 128 B), K8 half (64 rows x 128 B), V^T half (64 d x 128 B); a
       // K = 32 step advances 32 bytes inside the swizzle atom
@@ -721,7 +711,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                 tc_fence_after();
 #pragma unroll
                 for (int kk = 0; kk < 2 * kPSplit; ++kk)
-                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
               }
               __syncwarp();
             }
@@ -733,7 +723,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
               if (!kF8 && j + 2 < nkv) {
 #pragma unroll
                 for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
-                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
                 issue_s(d_s, qd, kd, false);
                 if (j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (qi & 1)), 3);
               } else {
@@ -745,7 +735,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                 } else {
 #pragma unroll
                   for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
-                    tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((2048u * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+                    tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
                 }
                 const bool s_next = j + 2 == nkv;
                 if (j + 2 < nkv || (s_next && nkv_next > 0 && ahead_next)) {

@@ -6,7 +6,7 @@
 //   smem descriptor: bits 0-13 start address >> 4, 16-29 leading-dimension
 //     byte offset >> 4, 32-45 stride-dimension byte offset >> 4, 46-47 = 1
 //     (descriptor version), 49-51 base offset (0: atoms are 1024-B aligned),
-//     52 LBO mode (0), 61-63 swizzle (2 = 128-byte swizzle).
+//     52 LBO mode (0), 61-63 swizzle (2 = 128-byte swizzle, 4 = 64-byte).
 //   instruction descriptor, kind::f16: bits 4-5 D format (1 = f32), 7-9 A
 //     format (1 = bf16), 10-12 B format (1 = bf16), 15 A major (0 = K), 16 B
 //     major (0 = K, 1 = MN), 17-22 N >> 3, 24-28 M >> 4.
@@ -332,6 +332,12 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t saddr, uint32_t lbo, ui
   return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) |
          (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) |
          (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (2ull << 61);
+}
+// The same with the 64-byte swizzle (atoms of 8 rows x 64 B).
+__device__ __forceinline__ uint64_t sdesc_sw64(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
+  return static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4) |
+         (static_cast<uint64_t>((lbo >> 4) & 0x3FFFu) << 16) |
+         (static_cast<uint64_t>((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46) | (4ull << 61);
 }
 
 // ---------------------------------------------------------------- scalar helpers

@@ -118,17 +118,19 @@ EncodeTiledFn encode_fn() {
 }
 
 // THD bf16 tensor [rows, H, D] seen as a 2-D array (H*D columns, rows rows);
-// box = 64 columns (128 bytes) x box_rows rows with the 128-byte swizzle.
-int make_tmap(CUtensorMap* m, const void* base, int64_t rows, int H, int D, uint32_t box_rows = 128) {
+// box = 64 columns (128 bytes) x box_rows rows with the 128-byte swizzle, or 32
+// columns with the 64-byte swizzle (a V half at head dim 64).
+int make_tmap(CUtensorMap* m, const void* base, int64_t rows, int H, int D, uint32_t box_rows = 128,
+              uint32_t box_cols = 64) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return fail(REFCACHE_ERR_CUDA, "cuTensorMapEncodeTiled is unavailable");
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(H) * D, static_cast<cuuint64_t>(std::max<int64_t>(rows, 1))};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(H) * D * 2};
-  const cuuint32_t box[2] = {64, box_rows};
+  const cuuint32_t box[2] = {box_cols, box_rows};
   const cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(REFCACHE_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", static_cast<int>(r));
   return REFCACHE_OK;
 }
@@ -376,19 +378,19 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
   // of tile / 2 rows, one per 64 head-dim columns) and a V box of the whole
   // tile.
   const uint32_t tile = static_cast<uint32_t>(tc2_tile(f8 != nullptr));
-  const uint32_t k_rows = tile / 2, v_rows = tile;
+  const uint32_t k_rows = tile / 2, v_rows = tile, v_cols = static_cast<uint32_t>(D / 2);
   CUtensorMap maps[5];
   int rc;
   if ((rc = make_tmap(&maps[0], op.q, op.q_rows, H, D)) != 0) return rc;
   if ((rc = make_tmap(&maps[1], op.ka, op.a_rows, H, D, k_rows)) != 0) return rc;
-  if ((rc = make_tmap(&maps[2], op.va, op.a_rows, H, D, v_rows)) != 0) return rc;
+  if ((rc = make_tmap(&maps[2], op.va, op.a_rows, H, D, v_rows, v_cols)) != 0) return rc;
   if (f8) {
     if ((rc = make_tmap_u8(&maps[3], f8->k8, static_cast<int64_t>(H) * D, f8->rows_pad)) != 0) return rc;
     if ((rc = make_tmap_u8(&maps[4], f8->vt8, f8->rows_pad, static_cast<int64_t>(H) * D)) != 0) return rc;
     a.b_scales = f8->scales;
   } else if (op.kb && op.b_rows > 0) {
     if ((rc = make_tmap(&maps[3], op.kb, op.b_rows, H, D, k_rows)) != 0) return rc;
-    if ((rc = make_tmap(&maps[4], op.vb, op.b_rows, H, D, v_rows)) != 0) return rc;
+    if ((rc = make_tmap(&maps[4], op.vb, op.b_rows, H, D, v_rows, v_cols)) != 0) return rc;
   } else {
     maps[3] = maps[1];
     maps[4] = maps[2];
