@@ -22,8 +22,7 @@
 // the 128-column O fit in the 512 TMEM columns; each handshake then carries
 // 1536 tensor cycles of MMAs instead of 1024 (see Cfg).
 //
-// Cluster of 2 CTAs (rank 0 = leader), 224 threads each (352 in the E4M3
-// kernel, whose 8 softmax warps split each row's columns, see below):
+// Cluster of 2 CTAs (rank 0 = leader), 224 threads each:
 //   warps 0-3  softmax: thread l of warp w owns row 32 w + l of this CTA's
 //              128 rows (its TMEM lane), all kBN score columns of a tile
 //   warp 4     TMA producer: this CTA's Q rows and its halves of the K and V
@@ -81,6 +80,8 @@
 //                      has finished reading O for the previous item.
 //   p_half[t % 2]      192-key tiles: the same for P's first 96 keys, whose
 //                      P.V MMAs are issued while the softmax works on the rest
+//                      (E4M3 kernel: 64 of 128 keys, with them S_t+2, since P has
+//                      buffers of its own there and S_t has been read by then)
 //   k_full[s] v_full[s]  the producers' TMA bytes of both CTAs (leader's barriers)
 //   q_full             per Q buffer, once per item
 //   q_empty            per Q buffer: the item's last S has read it, and the
@@ -137,8 +138,8 @@ namespace tc2 {
 using tc::Ctl;
 constexpr int kD = 128;
 constexpr uint32_t kQTile = 128 * 128 * 2;
-// Warp roles: softmax warps first (4, or 8 in the E4M3 kernel, two per SM
-// sub-partition), then the producer, the MMA warp and the gate warp.
+// Warp roles: softmax warps first, then the producer, the MMA warp and the gate
+// warp.
 //
 // kBN = keys per tile: 128, or 192 for the bf16 cache.  With 192-key tiles P
 // is written over the first half of its own S buffer, so that tensor memory
@@ -150,8 +151,7 @@ constexpr uint32_t kQTile = 128 * 128 * 2;
 template <bool kF8, int kBN>
 struct Cfg {
   static_assert(kBN == 128 || (kBN == 192 && !kF8), "key tiles of 128 keys, or 192 with the bf16 cache");
-  static constexpr int kHalves = kF8 ? 2 : 1;         // softmax warps per 32 rows
-  static constexpr int kSoftmaxWarps = 4 * kHalves;
+  static constexpr int kSoftmaxWarps = 4;
   static constexpr int kProducerWarp = kSoftmaxWarps, kMmaWarp = kSoftmaxWarps + 1, kGateWarp = kSoftmaxWarps + 2;
   static constexpr int kThreads = 32 * (kSoftmaxWarps + 3);
   static constexpr int kWarpArrivals = 2 * kSoftmaxWarps;  // p_full / q8_full: every softmax warp of both CTAs
@@ -170,7 +170,7 @@ struct Cfg {
   static constexpr uint32_t kColO = 384;
   // 32-key chunks of P handed over ahead of the rest (0: P in one piece), see
   // the head of the file
-  static constexpr int kPSplit = kPOverS ? 3 : 0;
+  static constexpr int kPSplit = kPOverS ? 3 : kF8 ? 2 : 0;
   static_assert(2 * kBN <= 384 && kColO + kD <= tc::kTmemCols, "tensor-memory layout");
 };
 constexpr int kPairDoneBars = 4;          // pair_done[g % 4]: a waiter for group g holds up group g + 4
@@ -189,11 +189,10 @@ struct SmemT {
   static constexpr uint32_t kRing = 2 * kQTile;    // slot s: [K half | V half]
   static constexpr uint32_t kQ8 = kRing + kStages * C::kStage;  // E4M3 Q tile (kF8 only)
   static constexpr uint32_t kScales = kQ8 + (kF8 ? kQ8Tile : 0u);  // ring of kScaleSlots x 16 B (kF8 only)
-  static constexpr uint32_t kLX = kScales + (kF8 ? kScaleSlots * 16u : 0u);  // [2][128] fp32 partial row sums
-  static constexpr uint32_t kBars = kLX + (kF8 ? 2u * 128u * 4u : 0u);
+  static constexpr uint32_t kBars = kScales + (kF8 ? kScaleSlots * 16u : 0u);
   static constexpr int kQFull = 0, kQEmpty = 2, kKFull = 4, kVFull = kKFull + kStages, kPairDone = kVFull + kStages,
                        kPFull = kPairDone + kPairDoneBars, kPHalf = kPFull + 2, kMmaDone = kPHalf + 2, kQ8Full = kMmaDone + 1,
-                       kLXFull = kQ8Full + 1, kScaleFull = kLXFull + 1, kScaleEmpty = kScaleFull + kScaleSlots,
+                       kScaleFull = kQ8Full + 1, kScaleEmpty = kScaleFull + kScaleSlots,
                        kItemFull = kScaleEmpty + kScaleSlots, kItemEmpty = kItemFull + kItemSlots,
                        kNumBars = kItemEmpty + kItemSlots;
   static constexpr uint32_t kTmemHolder = kBars + 8 * kNumBars;
@@ -345,7 +344,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     for (int s = 0; s < tc2::kPairDoneBars; ++s) mbar_init(bar(L::kPairDone + s), 1);
     mbar_init(bar(L::kMmaDone), 1);
     mbar_init(bar(L::kQ8Full), kWarpArrivals);
-    mbar_init(bar(L::kLXFull), Cfg::kSoftmaxWarps);
     for (int s = 0; s < tc2::kScaleSlots; ++s) {
       mbar_init(bar(L::kScaleFull + s), 1);
       mbar_init(bar(L::kScaleEmpty + s), Cfg::kSoftmaxWarps);
@@ -705,45 +703,52 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           uint64_t vd = vd0 + static_cast<uint64_t>(vslot) * (kStage >> 4), kd = slot_k(t0 + 2);
           uint32_t a_p = tmem + kColP + odd * kPStride, d_s = tmem + kColS + odd * kBN, acc0 = 0;
           for (j = 0; j < nkv; ++j, ++g) {
+            // P V of 32-key chunks [c0, c1) of P
+            auto issue_pv = [&](int c0, int c1) {
+              if (kF8 && j >= na) {
+                const uint64_t vd8 = vd + (vd80 - vd0);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                  if (kk >= c0 && kk < c1)
+                    tc2_mma_ts_f8(tmem + kColO, a_p + 8u * kk, vd8 + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : acc0);
+              } else {
+#pragma unroll
+                for (int kk = 0; kk < kBN / 16; ++kk)
+                  if (kk >= 2 * c0 && kk < 2 * c1)
+                    tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+              }
+            };
+            // S_j+2, of this item or the next
+            auto issue_next = [&]() {
+              if (!kF8 && j + 2 < nkv) {
+                issue_s(d_s, qd, kd, false);
+                if (j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (qi & 1)), 3);
+                return;
+              }
+              const bool s_next = j + 2 == nkv;
+              if (j + 2 < nkv || (s_next && nkv_next > 0 && ahead_next)) {
+                const int q = qi + (s_next ? 1 : 0);
+                issue_s(d_s, qdesc0 + ((static_cast<uint32_t>(q & 1) * kQTile) >> 4), kd, kF8 && !s_next && j + 2 >= na);
+                if (s_next ? nkv_next == 1 : j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (q & 1)), 3);
+              }
+            };
             if (kPSplit > 0) {  // P's first chunks
               if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
+              if (!Cfg::kPOverS && j + 2 == nkv) named();
               if (elect_one()) {
                 tc_fence_after();
-#pragma unroll
-                for (int kk = 0; kk < 2 * kPSplit; ++kk)
-                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
+                issue_pv(0, kPSplit);
+                if (!Cfg::kPOverS) issue_next();
               }
               __syncwarp();
             }
             if (bar_red_or(tc2::kGateBarrier, 64, false)) goto mma_done;
-            if (j + 2 == nkv) named();
+            if ((kPSplit == 0 || Cfg::kPOverS) && j + 2 == nkv) named();
             if (elect_one()) {
               tc_fence_after();
               // P.V first: with P over S, the S overwrites P_j
-              if (!kF8 && j + 2 < nkv) {
-#pragma unroll
-                for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
-                  tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
-                issue_s(d_s, qd, kd, false);
-                if (j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (qi & 1)), 3);
-              } else {
-                if (kF8 && j >= na) {
-                  const uint64_t vd8 = vd + (vd80 - vd0);
-#pragma unroll
-                  for (int kk = 0; kk < 4; ++kk)
-                    tc2_mma_ts_f8(tmem + kColO, a_p + 8u * kk, vd8 + ((32u * kk) >> 4), kIdesc8, kk > 0 ? 1u : acc0);
-                } else {
-#pragma unroll
-                  for (int kk = 2 * kPSplit; kk < kBN / 16; ++kk)
-                    tc2_mma_ts(tmem + kColO, a_p + 8u * kk, vd + ((kVStep * kk) >> 4), kIdescO, kk > 0 ? 1u : acc0);
-                }
-                const bool s_next = j + 2 == nkv;
-                if (j + 2 < nkv || (s_next && nkv_next > 0 && ahead_next)) {
-                  const int q = qi + (s_next ? 1 : 0);
-                  issue_s(d_s, qdesc0 + ((static_cast<uint32_t>(q & 1) * kQTile) >> 4), kd, kF8 && !s_next && j + 2 >= na);
-                  if (s_next ? nkv_next == 1 : j + 3 == nkv) tc2_commit_mc(bar(L::kQEmpty + (q & 1)), 3);
-                }
-              }
+              issue_pv(kPSplit, kBN / 32);
+              if (kPSplit == 0 || Cfg::kPOverS) issue_next();
               tc2_commit_mc(bar(L::kPairDone + (g & 3)), 3);
             }
             __syncwarp();
@@ -836,28 +841,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     }
   } else {
     // ------------------------------------------------------------ softmax (both CTAs)
-    // kH = 1: warp w (0-3) owns rows 32 w .. 32 w + 31 of this CTA's 128 rows
-    // (its TMEM lanes) and all kBN key columns.  kH = 2 (E4M3 kernel): warps w
-    // and w + 4 share those rows, warp w + 4 hh taking key columns and O
-    // columns [64 hh, 64 hh + 64), so that two warps per SM sub-partition share
-    // the exponentials.  Both read the whole S row, find the same row maximum
-    // and take the same rescale decisions; their partial row sums meet in the
-    // epilogue through shared memory.
-    constexpr int kH = Cfg::kHalves;
-    constexpr int kC = kBN / kH;  // key columns of this thread
-    constexpr int kOC = DG / kH;  // O columns of this thread
-    const int quarter = warp & 3, hh = warp >> 2;
-    const int col0 = hh * kC, ocol0 = hh * kOC;
-    const int trow = quarter * 32 + lane;                  // row within this CTA's 128 rows (= TMEM lane)
+    // Warp w (0-3) owns rows 32 w .. 32 w + 31 of this CTA's 128 rows (its TMEM
+    // lanes) and all kBN key columns.  (E4M3 kernel: two warps per row, each with
+    // half the columns, took the same time: both read the whole row for its
+    // maximum, and the two of a sub-partition take turns rather than overlap.)
+    const int trow = warp * 32 + lane;                     // row within this CTA's 128 rows (= TMEM lane)
     const int prow = 128 * static_cast<int>(rank) + trow;  // row within the item
-    const uint32_t lane_off = static_cast<uint32_t>(quarter * 32) << 16;
+    const uint32_t lane_off = static_cast<uint32_t>(warp * 32) << 16;
     const float sl2 = args.scale_log2;
     const f32x2 sl2x2 = make_f32x2(sl2, sl2);
-    float* lx = reinterpret_cast<float*>(base_ptr + L::kLX);  // [2][128] partial row sums (kH = 2)
     const uint32_t lp = lbar(0);  // the leader's barriers (mapped once)
     int t = 0;     // tiles of earlier items
     int G = 1;     // the item's group of S_1 (S_j: ready after group G + j - 1; P_j V_j: group G + 1 + j)
-    int n_lx = 0;  // row-sum exchanges so far (kH = 2)
     int si = 0;    // cached tiles read from the scale ring so far
     // wait until group g is complete (both CTAs see the multicast commit)
     auto wait_group = [&](int g, int where) -> bool {
@@ -874,10 +869,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       const int64_t grow = static_cast<int64_t>(tk.q_row0) + prow;
       if (nkv == 0) {
         if (row_ok) {
-          __nv_bfloat16* orow = args.out + grow * args.row_stride + static_cast<int64_t>(head) * DG + ocol0;
+          __nv_bfloat16* orow = args.out + grow * args.row_stride + static_cast<int64_t>(head) * DG;
           uint4 z = make_uint4(0, 0, 0, 0);
-          for (int c = 0; c < kOC / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = z;
-          if (args.lse && hh == 0) args.lse[grow * args.num_heads + head] = -INFINITY;
+          for (int c = 0; c < DG / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = z;
+          if (args.lse) args.lse[grow * args.num_heads + head] = -INFINITY;
         }
         __syncwarp();
         if (lane == 0) ring_done(k);
@@ -890,7 +885,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       if (kF8 && nkv > na) {
         // quantise this thread's query row of this head into the E4M3 Q tile:
         // s = amax / 448, code = E4M3(x * (448 / amax)), round to nearest even
-        // (the maximum over the whole row; each half writes its own columns)
         uint4 raw[16];
         if (row_ok) {
           const uint4* src = reinterpret_cast<const uint4*>(args.q + grow * args.row_stride + static_cast<int64_t>(head) * D);
@@ -912,7 +906,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         const uint32_t q8_row = base + L::kQ8 + static_cast<uint32_t>(trow) * 128u;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {  // 16 codes per 16-byte chunk, 128-byte swizzle
-          if (kH == 2 && (c >> 2) != hh) continue;
           uint32_t w[4];
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
@@ -934,6 +927,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         l2_ref = sc0.y > 0.f ? sc0.z : 0.f;
       }
       bool ready = false;  // this tile's S was seen ready at the end of the tile before
+      bool sc_ready = false;  // this cached tile's scales were read during the tile before
+      float4 sc_next = make_float4(0.f, 0.f, 0.f, 0.f);
       for (int j = 0; j < nkv; ++j, ++t) {
         const int b = t & 1;
         const int valid = (j < na ? tk.a_len : tk.b_len + na * kBN) - j * kBN;  // keys inside the range (>= kBN: all)
@@ -965,27 +960,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         // maximum sits on the latency loop that bounds the kernel (S ready ->
         // softmax -> P -> next S): with 96 max instructions per 192-key tile it
         // took about 190 of 2142 cycles.  Step at 4608 live and 20480 cached
-        // rows, 24 heads: 898 -> 838 us (E4M3 cache, where each half of a row
-        // finds the maximum of the whole row: 1040 -> 995 us), same bits.
-        float s[kC];
+        // rows, 24 heads: 898 -> 838 us, same bits.
+        float s[kBN];
         float m_raw;
         {
-          // with two halves, also the other half's columns, for the maximum only
           constexpr int kChains = kBN / 32;
           uint32_t r[kChains][32];
           float mx[kChains];
 #pragma unroll
-          for (int k = 0; k < kChains; ++k) {
-            const uint32_t col = static_cast<uint32_t>(kH == 1 ? 32 * k : (col0 + 32 * k) & (kBN - 1));
-            tmem_ld32_max(t_s + col, r[k], mx[k]);
-          }
+          for (int k = 0; k < kChains; ++k) tmem_ld32_max(t_s + 32u * k, r[k], mx[k]);
           if (t8) {
             // the producer's ring of tile scales (no global access here: an
             // ordinary load still in flight would hold up the next P arrival)
             const int sl = si % tc2::kScaleSlots;
-            if (!wait_warp(bar(L::kScaleFull + sl), static_cast<uint32_t>(si / tc2::kScaleSlots) & 1u, ctl, 17))
-              goto softmax_done;
-            const float4 sc = ld_shared_f4(base + L::kScales + 16u * static_cast<uint32_t>(sl));
+            if (!sc_ready) {
+              if (!wait_warp(bar(L::kScaleFull + sl), static_cast<uint32_t>(si / tc2::kScaleSlots) & 1u, ctl, 17))
+                goto softmax_done;
+              sc_next = ld_shared_f4(base + L::kScales + 16u * static_cast<uint32_t>(sl));
+            }
+            const float4 sc = sc_next;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(L::kScaleEmpty + sl));
             ++si;
@@ -999,7 +992,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
 #pragma unroll
           for (int k = 0; k < kChains; ++k) tmem_wait_ld(r[k], mx[k]);
 #pragma unroll
-          for (int k = 0; k < kC / 32; ++k)
+          for (int k = 0; k < kChains; ++k)
 #pragma unroll
             for (int c = 0; c < 32; ++c) s[32 * k + c] = __uint_as_float(r[k][c]);
           if constexpr (kChains == 6)
@@ -1016,9 +1009,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           const f32x2 alpha2 = make_f32x2(alpha, alpha);
           m_run = m_new;
           l_run *= alpha;
-          const uint32_t t_o = tmem + lane_off + kColO + static_cast<uint32_t>(ocol0);
-#pragma unroll
-          for (int cc = 0; cc < kOC / 16; ++cc) {
+          const uint32_t t_o = tmem + lane_off + kColO;
+          // (rolled in the E4M3 kernel: 919 -> 896 us at 4608 live and 20480 cached
+          // rows, 24 heads; the bf16 kernel is 0.5-1.5 % faster unrolled)
+          constexpr int kUnroll = kF8 ? 1 : DG / 16;
+#pragma unroll kUnroll
+          for (int cc = 0; cc < DG / 16; ++cc) {
             uint32_t o[16];
             tmem_ld16(t_o + 16u * cc, o);
             tmem_wait_ld(o);
@@ -1052,8 +1048,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
 #pragma unroll
           for (int i = 0; i < 4; ++i) lacc[i] = make_f32x2(0.f, 0.f);
           if (t8) {
+            // the next tile's scales are looked for and read on the way (waited for
+            // and read at its start they took 345 cycles of a tile's 1490: 967 us a
+            // step instead of 920)
+            const int sl = si % tc2::kScaleSlots;
+            bool found = false;
 #pragma unroll
-            for (int k = 0; k < kC / 32; ++k) {
+            for (int k = 0; k < kBN / 32; ++k) {
+              if (k == 0)
+                found = j + 1 < nkv &&
+                        mbar_test_wait(bar(L::kScaleFull + sl), static_cast<uint32_t>(si / tc2::kScaleSlots) & 1u);
+              if (k == 2 && found) sc_next = ld_shared_f4(base + L::kScales + 16u * static_cast<uint32_t>(sl));
               uint32_t pk[8];
 #pragma unroll
               for (int c = 0; c < 8; ++c) {
@@ -1067,11 +1072,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                 lacc[(2 * c + 1) & 3] = add_f32x2(lacc[(2 * c + 1) & 3], make_f32x2(x2, x3));
                 pk[c] = pack_e4m3x4(x0, x1, x2, x3);
               }
-              tmem_st8(t_p + static_cast<uint32_t>(col0 / 4) + 8u * k, pk);
+              tmem_st8(t_p + 8u * k, pk);
+              if (k == kPSplit - 1) p_arrive(L::kPHalf + b);
             }
+            sc_ready = __all_sync(0xffffffffu, found);
           } else {
 #pragma unroll
-            for (int k = 0; k < kC / 32; ++k) {
+            for (int k = 0; k < kBN / 32; ++k) {
               uint32_t pk[16];
 #pragma unroll
               for (int c = 0; c < 16; ++c) {
@@ -1082,7 +1089,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                 lacc[c & 3] = add_f32x2(lacc[c & 3], make_f32x2(x, y));
                 pk[c] = pack_bf16x2(x, y);
               }
-              tmem_st16(t_p + static_cast<uint32_t>(col0 / 2) + 16u * k, pk);
+              tmem_st16(t_p + 16u * k, pk);
               if (k == kPSplit - 1) p_arrive(L::kPHalf + b);
             }
           }
@@ -1117,26 +1124,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         if (lane == 0) ring_done(k);
         if (!wait_group(G + nkv, 10)) goto softmax_done;  // the item's last group
         tc_fence_after();
-        float l_tot = l_run;
-        if constexpr (kH == 2) {
-          // the two halves' partial row sums (relative to the same maximum)
-          lx[hh * 128 + trow] = l_run;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar(L::kLXFull));
-          if (!wait_warp(bar(L::kLXFull), static_cast<uint32_t>(n_lx) & 1u, ctl, 15)) goto softmax_done;
-          ++n_lx;
-          l_tot = l_run + lx[(1 - hh) * 128 + trow];
-        }
-        const float inv_l = kF8 ? s_ref / l_tot : 1.0f / l_tot;
-        const uint32_t t_o = tmem + lane_off + kColO + static_cast<uint32_t>(ocol0);
+        const float inv_l = kF8 ? s_ref / l_run : 1.0f / l_run;
+        const uint32_t t_o = tmem + lane_off + kColO;
         if (e_part > 0) {
           // a part of a split item: O / l in fp32 and m + log l to its workspace
           // slot, [D / 4][rows_per_task] float4, so that a warp's 32 rows of four
           // columns are one run of 512 bytes
           const int64_t slot = e_part - 1;
-          float4* dst = reinterpret_cast<float4*>(args.part_o) + (slot * (DG / 4) + ocol0 / 4) * args.rows_per_task + prow;
+          float4* dst = reinterpret_cast<float4*>(args.part_o) + slot * (DG / 4) * args.rows_per_task + prow;
 #pragma unroll
-          for (int cc = 0; cc < kOC / 32; ++cc) {
+          for (int cc = 0; cc < DG / 32; ++cc) {
             uint32_t o[32];
             tmem_ld32(t_o + 32u * cc, o);
             tmem_wait_ld(o);
@@ -1149,8 +1146,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
             }
           }
           tc_fence_before();
-          if (e_row_ok && hh == 0)
-            args.part_lse[slot * args.rows_per_task + prow] = (m_run + log2f(l_tot)) * 0.69314718055994530942f;
+          if (e_row_ok)
+            args.part_lse[slot * args.rows_per_task + prow] = (m_run + log2f(l_run)) * 0.69314718055994530942f;
         } else {
           // O / l as bf16 through the item's Q buffer, which its S no longer
           // reads: this thread's row in 16-byte chunks (swizzled), then whole
@@ -1158,12 +1155,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           // registers a warp's 16 bytes per row touch 32 lines per instruction,
           // 2048 cycles of the SM's load/store unit per item, which the next
           // item's softmax waited for.
-          constexpr int kNC = kOC / 8;                       // this thread's chunks of the row
-          constexpr uint32_t kPitch = 16u * kNC * kH;        // bytes of a staged row
-          const uint32_t stage = base + L::kQ + static_cast<uint32_t>(e_qb) * kQTile +
-                                 static_cast<uint32_t>(quarter * 32) * kPitch + static_cast<uint32_t>(hh) * 16u * kNC;
+          constexpr int kNC = DG / 8;              // chunks of a row
+          constexpr uint32_t kPitch = 16u * kNC;  // bytes of a staged row
+          const uint32_t stage = base + L::kQ + static_cast<uint32_t>(e_qb) * kQTile + static_cast<uint32_t>(warp * 32) * kPitch;
 #pragma unroll
-          for (int cc = 0; cc < kOC / 32; ++cc) {
+          for (int cc = 0; cc < DG / 32; ++cc) {
             uint32_t o[32];
             tmem_ld32(t_o + 32u * cc, o);
             tmem_wait_ld(o);
@@ -1184,9 +1180,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           __syncwarp();
           constexpr int kRows = 32 / kNC;  // rows per instruction
           const int r0 = lane / kNC, ch = lane % kNC;
-          const int first = 128 * static_cast<int>(rank) + quarter * 32;  // the warp's first row in the item
+          const int first = 128 * static_cast<int>(rank) + warp * 32;  // the warp's first row in the item
           __nv_bfloat16* dst = args.out + (static_cast<int64_t>(et.q_row0) + first) * args.row_stride +
-                               static_cast<int64_t>(e_head) * DG + ocol0 + 8 * ch;
+                               static_cast<int64_t>(e_head) * DG + 8 * ch;
 #pragma unroll 4
           for (int i = 0; i < kNC; ++i) {
             const int r = i * kRows + r0;
@@ -1194,8 +1190,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
                                          (static_cast<uint32_t>(ch ^ (r & (kNC - 1))) << 4));
             if (first + r < e_rows) *reinterpret_cast<uint4*>(dst + r * args.row_stride) = v;
           }
-          if (e_row_ok && args.lse && hh == 0)
-            args.lse[e_grow * args.num_heads + e_head] = (m_run + log2f(l_tot)) * 0.69314718055994530942f;
+          if (e_row_ok && args.lse)
+            args.lse[e_grow * args.num_heads + e_head] = (m_run + log2f(l_run)) * 0.69314718055994530942f;
         }
         // the Q buffer is free for the TMA loads of the item after the next
         fence_proxy_async_smem();
