@@ -437,22 +437,30 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
 // When a list of items, taken longest first by whichever of `clusters` CTA pairs
 // is free, is done (in key-tile times).  `costs`: how many items of each cost.
 double list_end(const std::map<double, int64_t, std::greater<double>>& costs, int clusters) {
-  std::vector<double> heap(static_cast<size_t>(clusters), 0.0);  // a min-heap of the pairs' end times
+  std::vector<double> ends(static_cast<size_t>(clusters), 0.0);  // when each pair is free, ascending
   for (const auto& [cost, n_items] : costs) {
     int64_t n = n_items;
-    // while the pairs' ends lie within one item of each other, the next `clusters`
-    // equal items go one to each
-    if (n >= clusters && *std::max_element(heap.begin(), heap.end()) - heap.front() <= cost) {
-      for (double& e : heap) e += cost * static_cast<double>(n / clusters);
-      n %= clusters;
-    }
-    for (; n > 0; --n) {
-      std::pop_heap(heap.begin(), heap.end(), std::greater<double>());
-      heap.back() += cost;
-      std::push_heap(heap.begin(), heap.end(), std::greater<double>());
+    while (n > 0) {
+      if (ends.back() - ends.front() > cost) {  // one item to the first pair
+        const double e = ends.front() + cost;
+        const auto at = std::lower_bound(ends.begin() + 1, ends.end(), e);
+        std::move(ends.begin() + 1, at, ends.begin());
+        *(at - 1) = e;
+        --n;
+        continue;
+      }
+      // the ends lie within one item of each other: whole rounds go to all pairs,
+      // what is left to the first ones
+      if (n >= clusters) {
+        for (double& e : ends) e += cost * static_cast<double>(n / clusters);
+        n %= clusters;
+      }
+      for (int64_t k = 0; k < n; ++k) ends[static_cast<size_t>(k)] += cost;
+      std::inplace_merge(ends.begin(), ends.begin() + n, ends.end());
+      n = 0;
     }
   }
-  return *std::max_element(heap.begin(), heap.end());
+  return ends.back();
 }
 
 // Per-item list of `tasks` x heads (head-major, as the kernels enumerate
@@ -481,9 +489,10 @@ void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, b
   int best_s = 1;
   if (rem > 0) {
     double best = 0.0;
+    std::map<double, int64_t, std::greater<double>> whole;
+    for (const Task& t : tasks) whole[key_tiles(t) + item_cost] += H;
     for (int cand : {1, 2, 3, 4, 6, 8}) {
-      std::map<double, int64_t, std::greater<double>> costs;
-      for (const Task& t : tasks) costs[key_tiles(t) + item_cost] += H;
+      auto costs = whole;
       int64_t parts = 0;
       for (int64_t i = n - rem; i < n; ++i) {
         const int nkv = key_tiles(tasks[static_cast<size_t>(i % n_tasks)]);
