@@ -770,7 +770,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         j = -1;
       }
     mma_done:
-      if (issued && lane == 0) {  // every MMA must finish before TMEM is freed
+      // Every MMA must finish before TMEM is freed.  A commit covers the MMAs of the
+      // thread that executes it, so the lane that elect.sync picks issues it too.
+      __syncwarp();
+      if (issued && elect_one()) {
         tc2_commit_mc(bar(L::kMmaDone), 1);
         drain_one(bar(L::kMmaDone), 0u, args.timeout_ns);
       }
