@@ -246,13 +246,20 @@ __device__ __forceinline__ int slot_of(int t) { return t % kStages; }
 template <int kStages>
 __device__ __forceinline__ uint32_t slot_parity(int t) { return static_cast<uint32_t>(t / kStages) & 1u; }
 
-// Bounded wait on a barrier that other CTAs arrive on.
+// Bounded wait on a barrier that other CTAs arrive on, for TMA bytes and tensor
+// memory (ordered by the copies' completion and the tcgen05 fences).
 __device__ __forceinline__ bool wait_cl(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
   return tc::wait_one(bar, parity, c, where);
 }
 __device__ __forceinline__ bool wait_cl_warp(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
   const bool ok = wait_cl(bar, parity, c, where);
   return __all_sync(0xffffffffu, ok);
+}
+// The same for what the other CTA wrote, or has read, with ordinary loads and
+// stores before it arrived (with release at cluster scope): the acquire has to
+// be at cluster scope too.  Once per item; the phase is complete after wait_cl.
+__device__ __forceinline__ bool wait_cl_acquire(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
+  return wait_cl(bar, parity, c, where) && mbar_try_wait_acquire_cluster(bar, parity);
 }
 // Work counter [next item, clusters done]: this cluster takes no more items; the
 // last cluster resets both words for the next launch, which reads them only
@@ -295,6 +302,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   constexpr int kPSplit = Cfg::kPSplit;
   using tc2::group_parity;
   using tc2::wait_cl;
+  using tc2::wait_cl_acquire;
   using tc2::wait_cl_warp;
   using tc2::kKHalf8;
   using tc2::kVHalf8;
@@ -395,10 +403,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   // wait until item k is in the ring / this warp (one lane) is done with it
   auto ring_wait = [&](int k, int where) -> bool {
     const uint32_t full = bar(L::kItemFull + k % tc2::kItemSlots), parity = static_cast<uint32_t>(k / tc2::kItemSlots) & 1u;
-    // (complete after wait_cl; once more for the acquire of the leader's writes)
-    return wait_cl(full, parity, ctl, where) && (leader || mbar_try_wait_acquire_cluster(full, parity));
+    return leader ? wait_cl(full, parity, ctl, where) : wait_cl_acquire(full, parity, ctl, where);
   };
-  auto ring_done = [&](int k) { mbar_arrive_cluster(lbar(L::kItemEmpty + k % tc2::kItemSlots)); };
+  // (release: the leader overwrites the slots of both CTAs once all have read them)
+  auto ring_done = [&](int k) { mbar_arrive_release_cluster(lbar(L::kItemEmpty + k % tc2::kItemSlots)); };
   // item `it` of the work list
   auto fetch_item = [&](int it, Task& t, int& head) {
     if (spans.n == 0) {
@@ -484,7 +492,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         } else {
           const int k = n_pub, s = k % tc2::kItemSlots;
           if (k >= tc2::kItemSlots &&
-              !wait_cl(bar(L::kItemEmpty + s), static_cast<uint32_t>(k / tc2::kItemSlots - 1) & 1u, ctl, 21))
+              !wait_cl_acquire(bar(L::kItemEmpty + s), static_cast<uint32_t>(k / tc2::kItemSlots - 1) & 1u, ctl, 21))
             return false;
           publish(k, pub_task, pub_head, pub_q & 1);
           pub_end = pub_head < 0;
@@ -820,7 +828,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         if (k_wait) ok = ok && wait_k(t + 2);
         // the first cached tile's S also needs the E4M3 Q tile of both CTAs
         if (kF8 && nkv > na && (j + 2 == na || (j == -1 && na == 0))) {
-          ok = ok && wait_cl_warp(bar(L::kQ8Full), static_cast<uint32_t>(q8i) & 1u, ctl, 14);
+          ok = ok && __all_sync(0xffffffffu, wait_cl_acquire(bar(L::kQ8Full), static_cast<uint32_t>(q8i) & 1u, ctl, 14));
           ++q8i;
         }
         if (j >= 0) {

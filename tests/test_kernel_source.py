@@ -41,3 +41,21 @@ def test_every_commit_is_issued_by_the_lane_that_issued_the_mmas():
     assert direct and all("elect_one()" in g and "lane ==" not in g for g in direct), direct
     done = code[code.index("mma_done:"):code.index("drain_one(bar(L::kMmaDone)")]
     assert "elect_one()" in done and "__syncwarp()" in done
+
+
+def test_waits_for_the_other_ctas_stores_and_reads_are_at_cluster_scope():
+    """The follower's E4M3 Q tile is written, and the item ring read, with
+    ordinary instructions: the arrivals release, and the leader's waits acquire,
+    at cluster scope (an mbarrier operation without a scope is at CTA scope)."""
+    code, ptx = _code("attn_tc2.cuh"), _code("ptx.cuh")
+    for name, op in (("mbar_arrive_release_cluster", "mbarrier.arrive.release.cluster"),
+                     ("mbar_try_wait_acquire_cluster", "try_wait.parity.acquire.cluster")):
+        assert op in ptx[ptx.index(name):][:400]
+    for line in code.splitlines():
+        if "mbar_arrive" in line and ("kQ8Full" in line or "kItemEmpty" in line):
+            assert "mbar_arrive_release_cluster" in line, line
+        if "wait_" in line and ("kQ8Full" in line or "kItemEmpty" in line):
+            assert "wait_cl_acquire" in line, line
+    assert sum("wait_cl_acquire" in line for line in code.splitlines()) >= 4
+    helper = code[code.index("bool wait_cl_acquire("):][:300]
+    assert "mbar_try_wait_acquire_cluster" in helper
