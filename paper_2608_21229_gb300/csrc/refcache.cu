@@ -918,7 +918,6 @@ int refcache_create(refcache_t** out, int num_layers, int mask_mode, const refca
   if (!bs.empty() && e == cudaSuccess)
     e = cudaMemcpy(h->d_build_slot, bs.data(), bs.size() * sizeof(Task), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, 256);
-  if (e == cudaSuccess) e = cudaDeviceSynchronize();  // zero before any stream's first launch
   if (e != cudaSuccess) {
     if (h->owns) cudaFree(h->mem);
     delete h;
@@ -928,6 +927,16 @@ int refcache_create(refcache_t** out, int num_layers, int mask_mode, const refca
     if (h->owns) cudaFree(h->mem);
     delete h;
     return rc;
+  }
+  // Every list and the zeroed counter are on the device before any stream's first
+  // launch: a copy from pageable memory may return before it has arrived, streams
+  // that do not block are not ordered behind it, and a launch reads its list
+  // before it waits for the kernel before it.
+  if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
+    if (h->owns) cudaFree(h->mem);
+    cudaFree(h->aux);
+    delete h;
+    return cuda_fail(e, "cudaDeviceSynchronize(work tables)");
   }
   h->built.assign(num_layers, 0);
   *out = h;

@@ -1,0 +1,61 @@
+/* Stand-ins for the CUDA runtime calls that refcache_create and refcache_destroy
+ * make, for tests of the host side without a GPU: "device" memory is host memory
+ * and every call that touches it is recorded.  Preloaded before libcudart. */
+#include <stdlib.h>
+#include <string.h>
+
+typedef int cudaError_t;
+enum { kMaxCalls = 256 };
+static char g_calls[kMaxCalls]; /* m(emcpy), s(et), d(evice synchronise) */
+static int g_n;
+static int g_fail_at = -1; /* the recorded call that fails */
+static long long g_live;   /* allocations not freed */
+
+static cudaError_t record(char c) {
+  if (g_n < kMaxCalls - 1) g_calls[g_n++] = c;
+  return g_n - 1 == g_fail_at ? 1 : 0;
+}
+const char* host_cudart_calls(void) { return g_calls; }
+long long host_cudart_live(void) { return g_live; }
+void host_cudart_reset(int fail_at) {
+  memset(g_calls, 0, sizeof g_calls);
+  g_n = 0;
+  g_fail_at = fail_at;
+}
+
+cudaError_t cudaGetDevice(int* d) { return *d = 0; }
+cudaError_t cudaSetDevice(int d) { return d != 0; }
+cudaError_t cudaDeviceGetAttribute(int* v, int attr, int dev) {
+  (void)dev;
+  /* cudaDevAttrMultiProcessorCount, ComputeCapabilityMajor, ComputeCapabilityMinor */
+  *v = attr == 16 ? 152 : attr == 75 ? 10 : attr == 76 ? 3 : 0;
+  return 0;
+}
+cudaError_t cudaMalloc(void** p, size_t n) {
+  *p = aligned_alloc(256, (n + 255) / 256 * 256 + 256);
+  if (*p) ++g_live;
+  return *p ? 0 : 2;
+}
+cudaError_t cudaFree(void* p) {
+  if (p) --g_live;
+  free(p);
+  return 0;
+}
+cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, int kind) {
+  (void)kind;
+  const cudaError_t e = record('m');
+  if (!e) memcpy(dst, src, n);
+  return e;
+}
+cudaError_t cudaMemset(void* p, int v, size_t n) {
+  const cudaError_t e = record('s');
+  if (!e) memset(p, v, n);
+  return e;
+}
+cudaError_t cudaDeviceSynchronize(void) { return record('d'); }
+cudaError_t cudaFuncSetAttribute(const void* f, int attr, int v) { return (void)f, (void)attr, (void)v, 0; }
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* cfg) {
+  (void)f, (void)cfg;
+  *n = 76;
+  return 0;
+}

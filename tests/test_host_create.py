@@ -1,0 +1,81 @@
+"""refcache_create without a GPU: the library's CUDA runtime calls go to
+host-memory stand-ins (tests/c/host_cudart.c), in a child process."""
+import json
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_2608_21229_gb300 import build as cbuild
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+CHILD = r"""
+import ctypes, json, sys
+sys.path.insert(0, {root!r})
+from paper_2608_21229_gb300 import refcache as rc
+cudart = ctypes.CDLL(None)
+cudart.host_cudart_calls.restype = ctypes.c_char_p
+cudart.host_cudart_live.restype = ctypes.c_longlong
+L = rc.load()
+
+
+def create(heads, dim, reqs, flags=0, fail_at=-1, tables=False):
+    # reqs: (anchor, instruction, target, reference) rows of each request
+    cu_l, cu_s = [0], [0]
+    for n_st, n_lt, n_x, n_r in reqs:
+        cu_l.append(cu_l[-1] + n_lt + n_x)
+        cu_s.append(cu_s[-1] + n_st + n_r)
+    seg = rc.Segments(heads, dim, cu_l, cu_s, [r[0] for r in reqs], [r[1] for r in reqs])
+    h = ctypes.c_void_p()
+    cudart.host_cudart_reset(fail_at)
+    code = L.refcache_create(ctypes.byref(h), 1, flags, ctypes.byref(seg.c), None, 0)
+    out = dict(code=code, calls=cudart.host_cudart_calls().decode(), live=cudart.host_cudart_live())
+    if code == 0:
+        out["step_launches"] = L.refcache_call_launches(h, 1)
+        L.refcache_destroy(h)
+    out["live_after"] = cudart.host_cudart_live()
+    return out
+
+
+{body}
+"""
+
+
+@pytest.fixture(scope="module")
+def run_child(tmp_path_factory):
+    shim = str(tmp_path_factory.mktemp("cudart") / "host_cudart.so")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-o", shim, os.path.join(ROOT, "tests", "c", "host_cudart.c")],
+                   check=True)
+    cbuild.build()
+
+    def run(body):
+        r = subprocess.run([sys.executable, "-c", CHILD.format(root=ROOT, body=body)], capture_output=True, text=True,
+                           timeout=300, env=dict(os.environ, LD_PRELOAD=shim))
+        assert r.returncode == 0, r.stderr
+        return json.loads(r.stdout.splitlines()[-1])
+
+    return run
+
+
+@pytest.mark.parametrize("flags", [0, 0x100])
+def test_create_returns_only_after_its_lists_are_on_the_device(run_child, flags):
+    """A host-to-device copy from pageable memory may return before it has
+    reached the device, and a non-blocking stream is not ordered behind it: a
+    launch reads its work list before it waits for anything, so the device is
+    synchronised after the last upload."""
+    out = run_child(f"print(json.dumps(create(24, 128, [(64, 256, 1024, 20480)], {flags})))")
+    assert out["code"] == 0 and out["live_after"] == 0
+    calls = out["calls"]
+    last = max(calls.rindex("m"), calls.rindex("s"))
+    assert "d" in calls[last:], calls
+
+
+def test_create_gives_back_its_memory_when_a_call_fails(run_child):
+    out = run_child("""
+ok = create(24, 128, [(64, 256, 1024, 20480)])
+print(json.dumps([create(24, 128, [(64, 256, 1024, 20480)], 0, i) for i in range(len(ok["calls"].rstrip("d")) + 1)]))""")
+    assert len(out) >= 5
+    for r in out:
+        assert r["code"] != 0 and r["live_after"] == 0, r
