@@ -598,10 +598,14 @@ struct refcache {
   CopySeg* d_copy = nullptr;
   int n_copy = 0, n_copy_pieces = 0;
   // per-item lists of the pair kernel, ordered for the persistent
-  // grid (the step's with split items), in a separate allocation:
-  // [build items | step items | step jobs | part_o | part_lse]
+  // grid (the step's with split items), and its copy of the in-slot build's task
+  // list, in a separate allocation: a launch reads its list before it waits for
+  // the kernel before it, which may be one of the caller's that writes the cache's
+  // memory (restores it, say) where that is the caller's.
+  // [build items | step items | step jobs | in-slot build tasks | part_o | part_lse]
   uint8_t* aux = nullptr;
   ItemList build_items, step_items;
+  const Task* build_slot_list = nullptr;
   __nv_bfloat16* slots = nullptr;
   int64_t slot_elems = 0;
   // E4M3 cache (REFCACHE_CACHE_FP8): per layer [k8 | vt8 | scales] of
@@ -778,7 +782,8 @@ int check_ptrs(std::initializer_list<const void*> ps, int64_t rows, const char* 
 // prefill outputs depend on its own (N_ST, N_R) only -- not on the other
 // requests of the batch, nor on the device's SM count -- and the cached block
 // is reproduced bit for bit (Sec. 3.3).  Both are ordered by longest_first.
-int plan_split_items(refcache* h, DeviceInfo* info, const std::vector<Task>& bt, const std::vector<Task>& st) {
+int plan_split_items(refcache* h, DeviceInfo* info, const std::vector<Task>& bt, const std::vector<Task>& st,
+                     const std::vector<Task>& bs) {
   // planned for the step kernel selected now (key tiles of tc2_tile(); the
   // split and the order stay correct, only less even, if another tile size
   // or grid runs them)
@@ -809,6 +814,8 @@ int plan_split_items(refcache* h, DeviceInfo* info, const std::vector<Task>& bt,
   off = align_up(off + si.size() * sizeof(Task), 256);
   const size_t o_sj = off;
   off = align_up(off + sj.size() * sizeof(CombineJob), 256);
+  const size_t o_bs = off;
+  off = align_up(off + bs.size() * sizeof(Task), 256);
   const size_t o_po = off;
   off = align_up(off + static_cast<size_t>(parts) * rows * h->D * sizeof(float), 256);
   const size_t o_pl = off;
@@ -823,7 +830,8 @@ int plan_split_items(refcache* h, DeviceInfo* info, const std::vector<Task>& bt,
   };
   if ((e = put(o_bi, bi.data(), bi.size() * sizeof(Task))) != cudaSuccess ||
       (e = put(o_si, si.data(), si.size() * sizeof(Task))) != cudaSuccess ||
-      (e = put(o_sj, sj.data(), sj.size() * sizeof(CombineJob))) != cudaSuccess) {
+      (e = put(o_sj, sj.data(), sj.size() * sizeof(CombineJob))) != cudaSuccess ||
+      (e = put(o_bs, bs.data(), bs.size() * sizeof(Task))) != cudaSuccess) {
     cudaFree(h->aux);
     h->aux = nullptr;
     return cuda_fail(e, "cudaMemcpy(split work list)");
@@ -833,6 +841,7 @@ int plan_split_items(refcache* h, DeviceInfo* info, const std::vector<Task>& bt,
   h->step_items = ItemList{reinterpret_cast<Task*>(h->aux + o_si), static_cast<int>(si.size()),
                            reinterpret_cast<CombineJob*>(h->aux + o_sj), static_cast<int>(sj.size()),
                            reinterpret_cast<float*>(h->aux + o_po), reinterpret_cast<float*>(h->aux + o_pl)};
+  h->build_slot_list = reinterpret_cast<Task*>(h->aux + o_bs);
   return REFCACHE_OK;
 }
 
@@ -923,7 +932,7 @@ int refcache_create(refcache_t** out, int num_layers, int mask_mode, const refca
     delete h;
     return cuda_fail(e, "cudaMemcpy(work tables)");
   }
-  if ((rc = plan_split_items(h, info, bt, st)) != 0) {
+  if ((rc = plan_split_items(h, info, bt, st, bs)) != 0) {
     if (h->owns) cudaFree(h->mem);
     delete h;
     return rc;
@@ -1072,7 +1081,8 @@ int refcache_build_in_slot(refcache_t* h, int layer, const void* q_static, const
               o_static,
               lse_static,
               h->d_status, true, h->d_work};
-  rc = run_attention(h->d_build_slot, h->n_build_slot, h->H, h->D, op, softmax_scale, info,
+  const Task* list = g_kernel.load() == REFCACHE_KERNEL_MMA_SYNC ? h->d_build_slot : h->build_slot_list;
+  rc = run_attention(list, h->n_build_slot, h->H, h->D, op, softmax_scale, info,
                      static_cast<cudaStream_t>(stream));
   if (rc) return rc;
   h->built[layer] = 1;

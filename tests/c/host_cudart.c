@@ -1,6 +1,6 @@
-/* Stand-ins for the CUDA runtime calls that refcache_create and refcache_destroy
- * make, for tests of the host side without a GPU: "device" memory is host memory
- * and every call that touches it is recorded.  Preloaded before libcudart. */
+/* Stand-ins for the CUDA runtime calls of the library's host side, for tests of
+ * it without a GPU: "device" memory is host memory, every call that touches it is
+ * recorded, and a launch is recorded instead of run.  Preloaded before libcudart. */
 #include <stdlib.h>
 #include <string.h>
 
@@ -57,5 +57,40 @@ cudaError_t cudaFuncSetAttribute(const void* f, int attr, int v) { return (void)
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const void* cfg) {
   (void)f, (void)cfg;
   *n = 76;
+  return 0;
+}
+
+/* Launches: threads per block, and the work list of the CTA-pair kernel (the first
+ * member of its sixth parameter; null for the other kernels). */
+enum { kMaxLaunches = 64, kPairThreads = 224 };
+static struct {
+  unsigned threads;
+  const void* list;
+} g_launch[kMaxLaunches];
+static int g_launches;
+int host_cudart_launches(void) { return g_launches; }
+unsigned host_cudart_threads(int i) { return g_launch[i].threads; }
+const void* host_cudart_list(int i) { return g_launch[i].list; }
+
+struct config {
+  unsigned grid[3], block[3]; /* the first members of cudaLaunchConfig_t */
+};
+cudaError_t cudaLaunchKernelExC(const struct config* cfg, const void* f, void** args) {
+  (void)f;
+  if (cfg->grid[1] > 65535 || cfg->grid[2] > 65535) return 9; /* cudaErrorInvalidConfiguration */
+  if (g_launches < kMaxLaunches) {
+    g_launch[g_launches].threads = cfg->block[0];
+    g_launch[g_launches].list = cfg->block[0] == kPairThreads ? *(const void**)args[5] : NULL;
+  }
+  ++g_launches;
+  return 0;
+}
+cudaError_t cudaGetLastError(void) { return 0; }
+static int encode_tiled(void* map) { return memset(map, 0, 128), 0; }
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** p, unsigned version, unsigned long long flags,
+                                             int* found) {
+  (void)name, (void)version, (void)flags;
+  *p = (void*)encode_tiled;
+  *found = 0; /* cudaDriverEntryPointSuccess */
   return 0;
 }

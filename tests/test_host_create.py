@@ -1,4 +1,4 @@
-"""refcache_create without a GPU: the library's CUDA runtime calls go to
+"""The library's host side without a GPU: its CUDA runtime calls go to
 host-memory stand-ins (tests/c/host_cudart.c), in a child process."""
 import json
 import os
@@ -18,17 +18,21 @@ from paper_2608_21229_gb300 import refcache as rc
 cudart = ctypes.CDLL(None)
 cudart.host_cudart_calls.restype = ctypes.c_char_p
 cudart.host_cudart_live.restype = ctypes.c_longlong
+cudart.host_cudart_list.restype = ctypes.c_void_p
 L = rc.load()
 
 
-def create(heads, dim, reqs, flags=0, fail_at=-1, tables=False):
+def segments(heads, dim, reqs):
     # reqs: (anchor, instruction, target, reference) rows of each request
     cu_l, cu_s = [0], [0]
     for n_st, n_lt, n_x, n_r in reqs:
         cu_l.append(cu_l[-1] + n_lt + n_x)
         cu_s.append(cu_s[-1] + n_st + n_r)
-    seg = rc.Segments(heads, dim, cu_l, cu_s, [r[0] for r in reqs], [r[1] for r in reqs])
-    h = ctypes.c_void_p()
+    return rc.Segments(heads, dim, cu_l, cu_s, [r[0] for r in reqs], [r[1] for r in reqs])
+
+
+def create(heads, dim, reqs, flags=0, fail_at=-1):
+    seg, h = segments(heads, dim, reqs), ctypes.c_void_p()
     cudart.host_cudart_reset(fail_at)
     code = L.refcache_create(ctypes.byref(h), 1, flags, ctypes.byref(seg.c), None, 0)
     out = dict(code=code, calls=cudart.host_cudart_calls().decode(), live=cudart.host_cudart_live())
@@ -79,3 +83,23 @@ print(json.dumps([create(24, 128, [(64, 256, 1024, 20480)], 0, i) for i in range
     assert len(out) >= 5
     for r in out:
         assert r["code"] != 0 and r["live_after"] == 0, r
+
+
+@pytest.mark.parametrize("dim", [64, 128])
+def test_lists_that_are_read_early_lie_in_the_librarys_own_memory(run_child, dim):
+    """The pair kernel reads a cache's work list before it waits for the kernel
+    before it, which may be one of the caller's that restores the cache memory it
+    owns: the list must not lie there."""
+    out = run_child(f"""
+seg, h, mem = segments(24, {dim}, [(64, 256, 1024, 2048), (3, 5, 70, 300)]), ctypes.c_void_p(), ctypes.c_void_p()
+n = L.refcache_bytes(1, 0, ctypes.byref(seg.c))
+assert cudart.cudaMalloc(ctypes.byref(mem), ctypes.c_size_t(n)) == 0
+assert L.refcache_create(ctypes.byref(h), 1, 0, ctypes.byref(seg.c), mem, n) == 0
+t = ctypes.c_void_p(1 << 20)
+calls = [L.refcache_build(h, 0, t, t, t, t, None, 0.1, None), L.step_attention(h, 0, t, t, t, t, None, 0.1, None),
+         L.refcache_build_in_slot(h, 0, t, t, t, t, None, 0.1, None)]
+lists = [cudart.host_cudart_list(i) for i in range(cudart.host_cudart_launches())]
+print(json.dumps(dict(calls=calls, mem=[mem.value, n], lists=[x for x in lists if x])))""")
+    assert out["calls"] == [0, 0, 0] and len(out["lists"]) == 3
+    lo, n = out["mem"]
+    assert not any(lo <= x < lo + n for x in out["lists"])
