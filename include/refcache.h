@@ -50,8 +50,13 @@
  *     concurrently.  Calls for different caches may run concurrently.
  *   - The tcgen05 attention kernel and the merge of split items are
  *     launched as programmatic dependents of the previous kernel on the
- *     stream: they wait for it to complete before they read memory, and they
- *     allow the kernel after them to start early.  A caller's kernel launched
+ *     stream: they wait for it to complete before they read any of the caller's
+ *     tensors or the cached K and V (they may read their own work lists, which
+ *     were complete when the cache was created, before that), and they
+ *     allow the kernel after them to start early.  The cache write of
+ *     refcache_build, launched behind the prefill in the same way, overlaps its
+ *     tail: it starts once every block of the prefill runs, and so has waited,
+ *     and ends after it.  A caller's kernel launched
  *     with programmatic stream serialization after a library call must
  *     therefore wait for its grid dependencies (griddepcontrol.wait) before it
  *     reads the library's outputs; ordinary launches need nothing.

@@ -446,7 +446,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   }
   // launched as a programmatic dependent of the previous kernel on the stream:
   // everything above overlaps its tail, nothing below reads memory before it
-  // is complete; and the next kernel may start its CTAs (they wait likewise)
+  // is complete; and the next kernel may start its CTAs (they wait likewise).
+  // The second line must stay behind the first: the cache writes read the static
+  // K and V and write the cache without a wait of their own, on the ground that
+  // every CTA of the prefill has passed this one.
   grid_dependency_wait();
   if (threadIdx.x == 0) grid_launch_dependents();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_holder, 0);

@@ -59,3 +59,13 @@ def test_waits_for_the_other_ctas_stores_and_reads_are_at_cluster_scope():
     assert sum("wait_cl_acquire" in line for line in code.splitlines()) >= 4
     helper = code[code.index("bool wait_cl_acquire("):][:300]
     assert "mbar_try_wait_acquire_cluster" in helper
+
+
+def test_the_kernel_behind_may_start_only_after_the_wait_for_the_one_before():
+    """The cache writes, dependents of the prefill, start on its triggers and wait
+    for nothing themselves before they write the cache: so a CTA triggers only
+    after its own wait, on every path."""
+    code = _code("attn_tc2.cuh")
+    kernel = code[code.index("attn_tc2_kernel("):]
+    assert kernel.count("grid_dependency_wait()") == 1 and kernel.count("grid_launch_dependents()") == 1
+    assert kernel.index("grid_dependency_wait()") < kernel.index("grid_launch_dependents()")
