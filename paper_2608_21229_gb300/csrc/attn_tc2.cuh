@@ -197,12 +197,12 @@ struct SmemT {
                        kNumBars = kItemEmpty + kItemSlots;
   static constexpr uint32_t kTmemHolder = kBars + 8 * kNumBars;
   static constexpr uint32_t kAbort = kTmemHolder + 4;
-  // load record of each CTA of the pair (leader's copy read at teardown):
-  // per CTA [loads per slot of the K and V rings (kRings) | own bytes of the
-  // last load per slot (kRings) | the other CTA's bytes of that load (kRings)
-  // | loads per Q buffer (2)]
-  static constexpr int kRings = 2 * kStages;
-  static constexpr uint32_t kRecWords = 3 * kRings + 2;
+  // load record of each CTA of the pair (leader's copy read at teardown): K
+  // tiles, V tiles and Q tiles loaded, whether the last K load of slot s (bit s)
+  // and the last V load (bit kStages + s) was of a cached E4M3 tile, and whether
+  // K tile 0 was left out (fault injection)
+  static constexpr int kRecK = 0, kRecV = 1, kRecQ = 2, kRecLast8 = 3, kRecSkipped = 4;
+  static constexpr uint32_t kRecWords = 5;
   static constexpr uint32_t kLoadRec = kAbort + 4;
   // ring of items: slot k % kItemSlots holds item k of this cluster (a Task;
   // head -1: none left); the gate warp passes the MMA warp its item's tiles
@@ -460,20 +460,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     // and K_t+2, which may belong to the next item, so that an item's first
     // loads are in flight before the item before it ends.
     if (lane == 0) {
-      // loads this CTA issued per K slot, V slot and Q buffer, and both CTAs'
-      // bytes of the last load of each slot; the leader arms every phase for
-      // both CTAs' bytes right before it issues its own half
-      int n_ring[L::kRings];
-      uint32_t own_bytes[L::kRings], other_bytes[L::kRings];
-      for (int s = 0; s < L::kRings; ++s) {
-        n_ring[s] = 0;
-        own_bytes[s] = 0;
-        other_bytes[s] = 0;
-      }
-      int n_q[2] = {0, 0};
-      int scale_armed[tc2::kScaleSlots];
-      for (int s = 0; s < tc2::kScaleSlots; ++s) scale_armed[s] = -1;
-      bool skip_next = leader && args.dbg_skip_first_load != 0;
+      // K and V tiles loaded (Q tiles: qi, scales: si), from which the loads of
+      // every slot follow, and the kind of the last load of each slot; the leader
+      // arms every phase for both CTAs' bytes right before it issues its own half.
+      // (Kept per slot, in arrays, they lay in local memory, at hundreds of cycles
+      // an access: the E4M3 kernel's producer took 11000 cycles from its last load
+      // to its end and held up the pair's.  Step with 256 live and 256 cached rows,
+      // 4 heads, E4M3: 21.4 us; now 9.7.  4608 and 20480, 24 heads: 911; now 892.)
+      int nk = 0, nv = 0;
+      uint32_t last8 = 0;
+      const bool skip = leader && args.dbg_skip_first_load != 0;
       int si = 0;  // cached tiles whose scales went into the ring
       // The leader's choice of the next item, in three steps, each of whose
       // result is first used by the following one: its index, its Task, its
@@ -542,9 +538,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           const uint32_t dst = base + L::kRing + static_cast<uint32_t>(slot) * kStage + kKHalf;
           const uint32_t full = lbar(L::kVFull + slot);
           if (leader) mbar_arrive_expect_tx(bar(L::kVFull + slot), 2 * vb);
-          ++n_ring[kStages + slot];
-          own_bytes[kStages + slot] = vb;
-          other_bytes[kStages + slot] = vb;
+          ++nv;
+          if (kF8) last8 = (last8 & ~(1u << (kStages + slot))) | (v8 ? 1u << (kStages + slot) : 0u);
           // head-dim columns [DG/2 r, DG/2 (r + 1)) of all kBN keys (E4M3: these
           // rows of V^T, all 128 keys)
           const int d0 = vt.head * DG + DG / 2 * static_cast<int>(rank);
@@ -572,7 +567,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           const uint32_t n = static_cast<uint32_t>(qi >> 1);
           if (!wait_one(bar(L::kQEmpty + b), (n & 1u) ^ 1u, ctl, 1)) goto producer_done;
           if (leader) mbar_arrive_expect_tx(bar(L::kQFull + b), 2 * kQBoxes * kBoxBytes);
-          ++n_q[b];
           const uint32_t qfull = lbar(L::kQFull + b);
           for (int ch = 0; ch < kQBoxes; ++ch)
             tma_load_2d_pair(base + L::kQ + b * kQTile + ch * kBoxBytes, &tm_q, qfull, kt.head * DG + ch * 64,
@@ -591,23 +585,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           const int sl = si % tc2::kScaleSlots, use = si / tc2::kScaleSlots;
           if (use > 0 && !wait_one(bar(L::kScaleEmpty + sl), static_cast<uint32_t>(use - 1) & 1u, ctl, 16)) break;
           mbar_arrive_expect_tx(bar(L::kScaleFull + sl), 16u);
-          scale_armed[sl] = use & 1;
           bulk_load(base + L::kScales + 16u * static_cast<uint32_t>(sl),
                     args.b_scales + ((kt.b_row0 >> 7) + (kj - k_na)) * args.num_heads + kt.head, 16u,
                     bar(L::kScaleFull + sl));
           ++si;
         }
         ++kj;
-        if (skip_next) {  // fault injection: the leader never arms or loads this tile
-          skip_next = false;
-          continue;
-        }
+        if (nk++ == 0 && skip) continue;  // fault injection: the leader never arms or loads this tile
         const uint32_t dst = base + L::kRing + static_cast<uint32_t>(slot) * kStage;
         const uint32_t full = lbar(L::kKFull + slot);
         if (leader) mbar_arrive_expect_tx(bar(L::kKFull + slot), 2 * kb);
-        ++n_ring[slot];
-        own_bytes[slot] = kb;
-        other_bytes[slot] = kb;
+        if (kF8) last8 = (last8 & ~(1u << slot)) | (k8 ? 1u << slot : 0u);
         // E4M3: keys [64 r, 64 r + 64), one box of 64 rows x 128 bytes; bf16: keys
         // [kBN/2 r, kBN/2 (r + 1)) of the tile, a box per 64 head-dim columns
         const void* map = ks.in_b ? &tm_kb : &tm_ka;
@@ -616,20 +604,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         if (kQBoxes == 2 && !k8) tma_load_2d_pair(dst + kKBox, map, full, kt.head * DG + 64, row);
       }
     producer_done:
-      // the scale ring's barriers are this CTA's own
-      for (int s = 0; s < tc2::kScaleSlots; ++s)
-        if (scale_armed[s] >= 0) drain_one(bar(L::kScaleFull + s), static_cast<uint32_t>(scale_armed[s]), args.timeout_ns);
+      // the scale ring's barriers are this CTA's own: the last load of each slot
+#pragma unroll 1
+      for (int s = 0; s < min(si, tc2::kScaleSlots); ++s)
+        drain_one(bar(L::kScaleFull + s), static_cast<uint32_t>((si - 1 - s) / tc2::kScaleSlots) & 1u, args.timeout_ns);
       // K, V and Q loads of both CTAs complete on the leader's barriers: record
       // this CTA's loads in the leader's shared memory, where the leader
       // settles and drains them after the teardown's first cluster barrier
       const uint32_t rec = mapa_shared(base + L::kLoadRec + rank * (L::kRecWords * 4u), 0);
-      for (int s = 0; s < L::kRings; ++s) {
-        st_cluster_u32(rec + 4u * s, static_cast<uint32_t>(n_ring[s]));
-        st_cluster_u32(rec + 4u * (L::kRings + s), own_bytes[s]);
-        st_cluster_u32(rec + 4u * (2 * L::kRings + s), other_bytes[s]);
-      }
-      st_cluster_u32(rec + 4u * (3 * L::kRings), static_cast<uint32_t>(n_q[0]));
-      st_cluster_u32(rec + 4u * (3 * L::kRings + 1), static_cast<uint32_t>(n_q[1]));
+      st_cluster_u32(rec + 4u * L::kRecK, static_cast<uint32_t>(nk));
+      st_cluster_u32(rec + 4u * L::kRecV, static_cast<uint32_t>(nv));
+      st_cluster_u32(rec + 4u * L::kRecQ, static_cast<uint32_t>(qi));
+      st_cluster_u32(rec + 4u * L::kRecLast8, last8);
+      st_cluster_u32(rec + 4u * L::kRecSkipped, skip && nk > 0 ? 1u : 0u);
       // this cluster takes no more items
       if (dyn && leader) tc2::work_done(args.work, n_clusters);
     }
@@ -1254,13 +1241,22 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       }
       if (mine > 0) drain_one(b, static_cast<uint32_t>(mine - 1) & 1u, args.timeout_ns);
     };
-    for (int s = 0; s < L::kRings; ++s)  // K slots, then V slots
-      settle(bar(L::kKFull + s), static_cast<int>(rec[s]), static_cast<int>(peer[s]), rec[2 * L::kRings + s],
-             peer[L::kRings + s]);
+    // loads of slot s of n, among `tiles` tiles
+    auto loads = [](uint32_t tiles, int s, int n) { return (static_cast<int>(tiles) - s + n - 1) / n; };
+    auto bytes = [&](const volatile uint32_t* r, int i, uint32_t full, uint32_t cached) {
+      return kF8 && (r[L::kRecLast8] >> i & 1u) ? cached : full;
+    };
+#pragma unroll 1
+    for (int s = 0; s < kStages; ++s) {
+      settle(bar(L::kKFull + s), loads(rec[L::kRecK], s, kStages) - (s == 0 && rec[L::kRecSkipped] ? 1 : 0),
+             loads(peer[L::kRecK], s, kStages), bytes(rec, s, kKBox * kQBoxes, kKHalf8),
+             bytes(peer, s, kKBox * kQBoxes, kKHalf8));
+      settle(bar(L::kVFull + s), loads(rec[L::kRecV], s, kStages), loads(peer[L::kRecV], s, kStages),
+             bytes(rec, kStages + s, kVHalf, kVHalf8), bytes(peer, kStages + s, kVHalf, kVHalf8));
+    }
     constexpr uint32_t kQCta = kQBoxes * kBoxBytes;  // each CTA's bytes of a Q load
     for (int b = 0; b < 2; ++b)
-      settle(bar(L::kQFull + b), static_cast<int>(rec[3 * L::kRings + b]), static_cast<int>(peer[3 * L::kRings + b]),
-             kQCta, kQCta);
+      settle(bar(L::kQFull + b), loads(rec[L::kRecQ], b, 2), loads(peer[L::kRecQ], b, 2), kQCta, kQCta);
   }
   // the follower leaves only once the leader has seen every load of the pair land
   cluster_sync();

@@ -3,6 +3,9 @@ matters after a wait has run out, and orderings between the two CTAs of a pair
 that hold on one machine by chance."""
 import os
 import re
+import subprocess
+
+from paper_2608_21229_gb300 import build as cbuild
 
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2608_21229_gb300", "csrc")
 
@@ -69,3 +72,14 @@ def test_the_kernel_behind_may_start_only_after_the_wait_for_the_one_before():
     kernel = code[code.index("attn_tc2_kernel("):]
     assert kernel.count("grid_dependency_wait()") == 1 and kernel.count("grid_launch_dependents()") == 1
     assert kernel.index("grid_dependency_wait()") < kernel.index("grid_launch_dependents()")
+
+
+def test_pair_kernel_keeps_no_arrays_in_local_memory(tmp_path):
+    """The roles' state lives in registers: an array indexed at run time goes to
+    local memory, where the producer of the E4M3 kernel spent more time than a
+    small step takes.  (A spilled register or two is no such array.)"""
+    cmd = cbuild.nvcc_cmd(str(tmp_path / "x.so"), ["-Xptxas", "-v"])
+    log = subprocess.run(cmd, capture_output=True, text=True, check=True).stderr
+    frames = dict(re.findall(r"Function properties for (\S*attn_tc2_kernel\S*)\s+(\d+) bytes stack frame", log))
+    assert len(frames) == 5, sorted(frames)
+    assert all(int(n) <= 16 for n in frames.values()), frames
