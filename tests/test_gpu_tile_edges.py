@@ -126,3 +126,24 @@ def test_e4m3_cache_write_at_the_edges_of_row_groups(mode, heads):
         t[w.cu_static[3]:w.cu_static[4]] = 0
     rcb.set_kernel("tcgen05")
     fp8.check_cache(fp8.Fp8Run(w, mode=mode, static=tuple(static)), np.arange(heads))
+
+
+@pytest.mark.parametrize("batch", [1, 2, 31, 32, 33, 34, 1024, 1025, 1100])
+def test_cache_write_finds_the_segment_of_every_piece(batch):
+    """The bf16 cache write of many requests, some without cached rows: the slots hold the rows' bytes."""
+    heads, dim = 3, 64  # rows of 384 bytes: segments of one piece, and of several with a short last one
+    lens = [0 if i % 7 == 5 else 1 + (i * 53) % 29 for i in range(batch)]
+    reqs = tuple(workloads.Request(i % 2, 0, 1, n) for i, n in enumerate(lens))
+    w = workloads.Workload("segments", heads, dim, reqs, 36)
+    seg = rcb.Segments.from_workload(w)
+    cache = rcb.RefCache(seg)
+    for t in cache.kv(0):
+        t.fill_(float("nan"))
+    q, k, v = (torch.randn(seg.static_rows, heads, dim, device="cuda", generator=torch.Generator("cuda").manual_seed(s)).to(torch.bfloat16)
+               for s in (7, 8, 9))
+    cache.build(0, q, k, v, torch.empty_like(q))
+    assert rcb.status() == rcb.OK, rcb.last_error()
+    rows = np.concatenate([np.arange(s + r.n_st, s + r.n_static) for s, r in zip(w.cu_static, reqs)])
+    rows = torch.from_numpy(rows).cuda()
+    for slot, t in zip(cache.kv(0), (k, v)):
+        assert torch.equal(slot.view(torch.int16), t[rows].view(torch.int16))
