@@ -24,33 +24,57 @@ namespace rc {
 constexpr int kMaxParts = 8;
 constexpr int kCombineRows = 32;
 
-// grid = (ceil(rows / 32), jobs), 256 threads: lane = row, warp w takes the
-// column quads w, w + 8, ...
-template <int D>
+// grid = (ceil(rows / 32), jobs, D / (32 kQ)), 256 threads: lane = row, kQ column
+// quads per thread.
+//
+// Two forms.  Few jobs leave the SMs idle and wait for memory, part after part: with
+// kAhead all parts' loads are in flight before the first is used, and a block takes
+// 64 columns.  Many jobs are bound by the L2's bandwidth and by the number of blocks
+// that fit on an SM (57 registers against 92): a block takes all columns, part after
+// part.  us a call, back to back, 256 rows of 128 columns, ahead / part after part:
+//   jobs     2 parts       4 parts        8 parts
+//      4   2.0 /  2.7    2.1 /  3.4     2.4 /  4.4
+//     12   2.3 /  2.7    2.4 /  3.5     2.8 /  4.5
+//     18   2.4 /  2.8    2.5 /  3.6     3.0 /  4.6
+//     24   3.7 /  2.9    3.9 /  3.7     4.8 /  4.9
+//     76   7.5 /  3.9    8.2 /  5.0    10.5 /  7.1
+// (Step with 256 live and 8192 cached rows, 4 heads, 8 parts: 17.6 us part after
+// part, now 13.8; on an E4M3 cache 20.1, now 17.0.)
+// The line (launch_combine) lies where the blocks of the first form fill two per SM.
+template <int D, int kQ, bool kAhead>
 __global__ void __launch_bounds__(256) combine_parts_kernel(const CombineJob* __restrict__ jobs,
                                                             const float* __restrict__ part_o,
                                                             const float* __restrict__ part_lse, int rows_per_part,
                                                             __nv_bfloat16* __restrict__ out, float* __restrict__ lse,
                                                             int64_t row_stride, int num_heads) {
-  static_assert(D == 128 || D == 64, "four or two column quads per thread");
-  constexpr int kQ = D / 32;        // column quads of this thread
-  constexpr int kPitch = D + 8;     // bf16 elements of a staged row (16 bytes of padding)
+  static_assert(D % (32 * kQ) == 0, "eight warps of kQ column quads");
+  constexpr int kCols = 32 * kQ;     // columns of this block
+  constexpr int kPitch = kCols + 8;  // bf16 elements of a staged row (16 bytes of padding)
   __shared__ __align__(16) __nv_bfloat16 tile[kCombineRows * kPitch];
   const CombineJob job = jobs[blockIdx.y];  // written when the cache was created
   const int r0 = blockIdx.x * kCombineRows, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = r0 + lane;
+  const int r = r0 + lane, col0 = kCols * blockIdx.z;
   grid_dependency_wait();  // the attention kernel's parts are complete
   if (threadIdx.x == 0) grid_launch_dependents();
   if (r0 >= job.q_rows) return;
   const bool ok = r < job.q_rows;
   const int np = min(job.nparts, kMaxParts);
+  const float4* src = reinterpret_cast<const float4*>(part_o) +
+                      (static_cast<int64_t>(job.part0) * (D / 4) + col0 / 4 + warp) * rows_per_part + r;
+  auto load = [&](int p, int c) { return src[(static_cast<int64_t>(p) * (D / 4) + 8 * c) * rows_per_part]; };
   float w[kMaxParts];
-  float lmax = -INFINITY;
+  float4 ahead[kMaxParts][kQ];
 #pragma unroll
   for (int p = 0; p < kMaxParts; ++p) {
     w[p] = p < np && ok ? part_lse[static_cast<int64_t>(job.part0 + p) * rows_per_part + r] : -INFINITY;
-    lmax = fmaxf(lmax, w[p]);
+    if (kAhead && p < np && ok) {
+#pragma unroll
+      for (int c = 0; c < kQ; ++c) ahead[p][c] = load(p, c);
+    }
   }
+  float lmax = -INFINITY;
+#pragma unroll
+  for (int p = 0; p < kMaxParts; ++p) lmax = fmaxf(lmax, w[p]);
   float wsum = 0.f;
 #pragma unroll
   for (int p = 0; p < kMaxParts; ++p) {
@@ -60,14 +84,12 @@ __global__ void __launch_bounds__(256) combine_parts_kernel(const CombineJob* __
   float4 acc[kQ];
 #pragma unroll
   for (int c = 0; c < kQ; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
-  const float4* src = reinterpret_cast<const float4*>(part_o) +
-                      (static_cast<int64_t>(job.part0) * (D / 4) + warp) * rows_per_part + r;
 #pragma unroll
   for (int p = 0; p < kMaxParts; ++p) {
     if (p < np && ok) {
 #pragma unroll
       for (int c = 0; c < kQ; ++c) {
-        const float4 x = src[(static_cast<int64_t>(p) * (D / 4) + 8 * c) * rows_per_part];
+        const float4 x = kAhead ? ahead[p][c] : load(p, c);
         acc[c].x += w[p] * x.x, acc[c].y += w[p] * x.y, acc[c].z += w[p] * x.z, acc[c].w += w[p] * x.w;
       }
     }
@@ -80,15 +102,15 @@ __global__ void __launch_bounds__(256) combine_parts_kernel(const CombineJob* __
     packed.y = pack_bf16x2(acc[c].z * inv, acc[c].w * inv);
     *reinterpret_cast<uint2*>(&tile[lane * kPitch + 4 * (warp + 8 * c)]) = packed;
   }
-  if (lse && warp == 0 && ok)
+  if (lse && blockIdx.z == 0 && warp == 0 && ok)
     lse[(static_cast<int64_t>(job.q_row0) + r) * num_heads + job.head] = lmax + logf(wsum);
   __syncthreads();
-  constexpr int kNC = D / 8;  // 16-byte chunks of a row
+  constexpr int kNC = kCols / 8;  // 16-byte chunks of a row
   for (int i = threadIdx.x; i < kCombineRows * kNC; i += 256) {
     const int rr = i / kNC, ch = i % kNC;
     if (r0 + rr < job.q_rows)
       *reinterpret_cast<uint4*>(out + (static_cast<int64_t>(job.q_row0) + r0 + rr) * row_stride +
-                                static_cast<int64_t>(job.head) * D + 8 * ch) =
+                                static_cast<int64_t>(job.head) * D + col0 + 8 * ch) =
           *reinterpret_cast<const uint4*>(&tile[rr * kPitch + 8 * ch]);
   }
 }

@@ -342,6 +342,33 @@ int launch_cache_write(const CacheWrite& w, const DeviceInfo* info, cudaStream_t
   return REFCACHE_OK;
 }
 
+// The merge of split items, behind the attention kernel (its blocks wait for it).
+template <int D>
+int launch_combine(const ItemList& il, const AttnArgs& a, const DeviceInfo* info, cudaStream_t s) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>((a.rows_per_task + rc::kCombineRows - 1) / rc::kCombineRows),
+                     static_cast<unsigned>(il.n_jobs), D / 64);
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const float* po = il.part_o;
+  const float* pl = il.part_lse;
+  // few jobs: more blocks, each with all parts' loads in flight (see the kernel)
+  const bool ahead = static_cast<int64_t>(cfg.gridDim.x) * cfg.gridDim.y * cfg.gridDim.z <= 2 * info->num_sms;
+  if (!ahead) cfg.gridDim.z = 1;
+  cudaError_t e = ahead ? cudaLaunchKernelEx(&cfg, rc::combine_parts_kernel<D, 2, true>, il.jobs, po, pl, a.rows_per_task,
+                                             a.out, a.lse, a.row_stride, a.num_heads)
+                        : cudaLaunchKernelEx(&cfg, rc::combine_parts_kernel<D, D / 32, false>, il.jobs, po, pl,
+                                             a.rows_per_task, a.out, a.lse, a.row_stride, a.num_heads);
+  if (e == cudaSuccess) e = cudaGetLastError();
+  if (e != cudaSuccess) return cuda_fail(e, "combine_parts_kernel launch");
+  return REFCACHE_OK;
+}
+
 // `write` (the build's cache write, if any) runs beside the pair kernel,
 // launched right after it; with the mma.sync kernel it goes first.
 int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands& op, float scale, DeviceInfo* info,
@@ -411,26 +438,7 @@ int run_attention(const Task* d_tasks, int n_tasks, int H, int D, const Operands
     rc = tile == 128 ? launch_tc2<false, 128, 64>(maps, a, spans, info, s) : launch_tc2<false, 192, 64>(maps, a, spans, info, s);
   if (rc) return rc;
   if (write && (rc = launch_cache_write(*write, info, s, true)) != 0) return rc;
-  if (il && il->n_jobs > 0) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(static_cast<unsigned>((a.rows_per_task + rc::kCombineRows - 1) / rc::kCombineRows),
-                       static_cast<unsigned>(il->n_jobs));
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;  // its CTAs wait for the attention kernel
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    const float* po = static_cast<const float*>(il->part_o);
-    const float* pl = static_cast<const float*>(il->part_lse);
-    cudaError_t e = D == 128 ? cudaLaunchKernelEx(&cfg, rc::combine_parts_kernel<128>, il->jobs, po, pl, a.rows_per_task,
-                                                  a.out, a.lse, a.row_stride, H)
-                             : cudaLaunchKernelEx(&cfg, rc::combine_parts_kernel<64>, il->jobs, po, pl, a.rows_per_task,
-                                                  a.out, a.lse, a.row_stride, H);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_fail(e, "combine_parts_kernel launch");
-  }
+  if (il && il->n_jobs > 0) return D == 128 ? launch_combine<128>(*il, a, info, s) : launch_combine<64>(*il, a, info, s);
   return REFCACHE_OK;
 }
 

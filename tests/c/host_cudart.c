@@ -7,6 +7,10 @@
 typedef int cudaError_t;
 enum { kMaxCalls = 256 };
 static char g_calls[kMaxCalls]; /* m(emcpy), s(et), d(evice synchronise) */
+static struct {
+  const void* dst;
+  size_t n;
+} g_copy[kMaxCalls]; /* of the call of the same index, where it is a memcpy */
 static int g_n;
 static int g_fail_at = -1; /* the recorded call that fails */
 static long long g_live;   /* allocations not freed */
@@ -16,6 +20,8 @@ static cudaError_t record(char c) {
   return g_n - 1 == g_fail_at ? 1 : 0;
 }
 const char* host_cudart_calls(void) { return g_calls; }
+const void* host_cudart_copy_dst(int i) { return g_copy[i].dst; }
+size_t host_cudart_copy_bytes(int i) { return g_copy[i].n; }
 long long host_cudart_live(void) { return g_live; }
 void host_cudart_reset(int fail_at) {
   memset(g_calls, 0, sizeof g_calls);
@@ -43,6 +49,7 @@ cudaError_t cudaFree(void* p) {
 }
 cudaError_t cudaMemcpy(void* dst, const void* src, size_t n, int kind) {
   (void)kind;
+  g_copy[g_n].dst = dst, g_copy[g_n].n = n;
   const cudaError_t e = record('m');
   if (!e) memcpy(dst, src, n);
   return e;

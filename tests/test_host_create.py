@@ -18,7 +18,8 @@ from paper_2608_21229_gb300 import refcache as rc
 cudart = ctypes.CDLL(None)
 cudart.host_cudart_calls.restype = ctypes.c_char_p
 cudart.host_cudart_live.restype = ctypes.c_longlong
-cudart.host_cudart_list.restype = ctypes.c_void_p
+cudart.host_cudart_list.restype = cudart.host_cudart_copy_dst.restype = ctypes.c_void_p
+cudart.host_cudart_copy_bytes.restype = ctypes.c_size_t
 L = rc.load()
 
 
@@ -38,6 +39,11 @@ def create(heads, dim, reqs, flags=0, fail_at=-1):
     out = dict(code=code, calls=cudart.host_cudart_calls().decode(), live=cudart.host_cudart_live())
     if code == 0:
         out["step_launches"] = L.refcache_call_launches(h, 1)
+        # after the memset: the build's items, the step's, its merge jobs (if any), the in-slot build's tasks (if any)
+        if out["step_launches"] == 2:
+            i = out["calls"].index("s") + 3
+            jobs = (ctypes.c_int32 * (cudart.host_cudart_copy_bytes(i) // 4)).from_address(cudart.host_cudart_copy_dst(i))
+            out["jobs"] = [list(jobs[k:k + 5]) for k in range(0, len(jobs), 8)]  # q_row0, q_rows, head, part0, nparts
         L.refcache_destroy(h)
     out["live_after"] = cudart.host_cudart_live()
     return out
@@ -103,3 +109,19 @@ print(json.dumps(dict(calls=calls, mem=[mem.value, n], lists=[x for x in lists i
     assert out["calls"] == [0, 0, 0] and len(out["lists"]) == 3
     lo, n = out["mem"]
     assert not any(lo <= x < lo + n for x in out["lists"])
+
+
+@pytest.mark.parametrize("dim", [64, 128])
+def test_workloads_of_the_split_tests_are_split_as_they_say(run_child, dim):
+    import split_workloads
+
+    cases = split_workloads.cases(dim)
+    reqs = [(w.num_heads, [(r.n_st, r.n_lt, r.n_x, r.n_r) for r in w.requests]) for w, _, _ in cases]
+    for flags, want in ((0, 1), (0x100, 2)) if dim == 128 else ((0, 1),):
+        out = run_child(f"print(json.dumps([create(h, {dim}, r, {flags}) for h, r in {reqs}]))")
+        for c, o in zip(cases, out):
+            assert o["code"] == 0 and o["step_launches"] == 2, c[0].name
+            assert sorted({j[4] for j in o["jobs"]}) == c[want], c[0].name
+    # both forms of the merge: 16 blocks a job (8 at head dim 64), two of which fit on each of 152 SMs
+    jobs = [len(o["jobs"]) * 8 * dim // 64 for o in out]
+    assert min(jobs) <= 304 < max(jobs)
