@@ -280,11 +280,13 @@ def test_split_tail_items_sampled():
     parts merged by a combine kernel; on the headline case those are items of
     the last heads (head-major order)."""
     run = pu.GpuRun(workloads.EDIT_1024_5REF, kernel="tcgen05")
+    assert run.cache.launches("step") == 2
     pu.sampled_compare(run, seed=21, per_request=64, heads=[21, 22, 23])
 
 
 def test_split_tail_items_cfg_pair_sampled():
     run = pu.GpuRun(workloads.CFG_1024_5REF, kernel="tcgen05")
+    assert run.cache.launches("step") == 2
     pu.sampled_compare(run, seed=22, per_request=32, heads=[22, 23])
 
 
@@ -297,7 +299,7 @@ def test_call_launch_counts():
     seg = rcb.Segments.from_workload(w)
     cache = rcb.RefCache(seg, num_layers=1, mask_mode="beyond")
     rcb.set_kernel("tcgen05")
-    assert cache.launches("step") in (1, 2)
+    assert cache.launches("step") == 2
     assert cache.launches("build") == 2
     rcb.set_kernel("mma_sync")
     assert cache.launches("step") == 1 and cache.launches("build") == 2
@@ -348,6 +350,7 @@ def test_split_tail_items_full_compare():
     oracle, and the cache and prefill as well."""
     w = workloads.Workload("split_tail_768x3000", 8, 128, (workloads.Request(64, 256, 512, 3000),), 19)
     run = pu.GpuRun(w, mode="beyond", kernel="tcgen05")
+    assert run.cache.launches("step") == 2
     pu.full_compare(run)
 
 
