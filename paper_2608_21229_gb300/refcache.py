@@ -243,7 +243,7 @@ class RefCache:
     handed to refcache_create, so the library itself allocates nothing.
     """
 
-    _slots = None  # views of every layer's (K slot, V slot), laid out by the first kv()
+    _slots = None  # (first byte of layer 0's K slot in the cache memory, rows), once kv() has asked for it
 
     def __init__(self, seg: Segments, num_layers: int = 1, mask_mode: str = "beyond", device=None,
                  cache_dtype: str = "bf16"):
@@ -279,29 +279,25 @@ class RefCache:
 
     def kv(self, layer: int):
         """(K slot, V slot) of a layer as bf16 [cache_rows, H, D] views of the cache memory."""
-        if self._slots is not None and self.h is not None and type(layer) is int and 0 <= layer < self.num_layers:
-            k, v = self._slots[layer]
-            return k[:], v[:]
         import torch
 
-        k, v, rows = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_int64()
-        _check(load().refcache_kv_ptr(self.h, layer, ctypes.byref(k), ctypes.byref(v), ctypes.byref(rows)))
         H, D = self.seg.num_heads, self.seg.head_dim
-        n = rows.value * H * D * 2
-        base = self.mem.data_ptr()
+        # The slots of all layers lie one after the other, K before V, so one answer of
+        # the library serves every layer (asking takes half the call's time).  The views
+        # are made anew each time: one made under inference_mode or no_grad carries that
+        # with it and cannot be written to outside.
+        if self._slots is None or self.h is None or type(layer) is not int or not 0 <= layer < self.num_layers:
+            k, v, rows = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_int64()
+            _check(load().refcache_kv_ptr(self.h, layer, ctypes.byref(k), ctypes.byref(v), ctypes.byref(rows)))
+            self._slots = (k.value - self.mem.data_ptr() - 4 * layer * rows.value * H * D, rows.value)
+        first, rows = self._slots
+        n = rows * H * D * 2
 
-        def view(p):
-            off = p.value - base
-            return self.mem[off:off + n].view(torch.bfloat16).view(rows.value, H, D)
+        def view(off):
+            return self.mem[off:off + n].view(torch.bfloat16).view(rows, H, D)
 
-        # the slots of all layers lie one after the other, K before V: views of them
-        # are laid out once, and a later call takes its layer's (asking the library for
-        # the addresses and viewing the bytes took 16 us a call)
-        first = k.value - base - 2 * n * layer
-        slots = self.mem[first:first + 2 * n * self.num_layers].view(torch.bfloat16).view(
-            self.num_layers, 2, rows.value, H, D)
-        self._slots = [(slots[i, 0], slots[i, 1]) for i in range(self.num_layers)]
-        return view(k), view(v)
+        off = first + 2 * n * layer
+        return view(off), view(off + n)
 
     def fp8(self, layer: int):
         """E4M3 cache of a layer as views of the cache memory: (K codes uint8

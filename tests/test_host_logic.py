@@ -1,11 +1,14 @@
 """Host logic: the accounting the benchmark reports against the App. C model,
-and the seeded input generators."""
+the seeded input generators, and the binding's views of the cache."""
+import contextlib
+
 import pytest
 import torch
 
 import workloads
 from oracle import cost_model as cm
 from paper_2608_21229_gb300 import accounting as acc
+from paper_2608_21229_gb300 import refcache as rcb
 
 
 @pytest.mark.parametrize("w", [workloads.TINY, workloads.EDIT_512_2REF, workloads.EDIT_1024_5REF]
@@ -80,3 +83,49 @@ def test_guard_report_finds_planted_writes():
     full[g + 12] = pat                     # a partly matching element is written
     assert pu.guard_report(full, g, n, 4, pat)[2] == 1
     assert pu.guard_report(full, g, n, 2, pat)[2] == 2
+
+
+class _KvLibrary:
+    """refcache_kv_ptr of a cache of 3 layers with 5 rows, 2 heads of 64, 256 bytes into its memory."""
+
+    def __init__(self, base):
+        self.base = base
+
+    def refcache_kv_ptr(self, h, layer, k, v, rows):
+        if h is None or not 0 <= layer < 3:
+            return rcb.ERR_INVALID_ARG
+        n = 5 * 2 * 64 * 2
+        k._obj.value, v._obj.value, rows._obj.value = self.base + 256 + 2 * n * layer, self.base + 256 + 2 * n * layer + n, 5
+        return rcb.OK
+
+    def refcache_last_error(self, buf, n):
+        return 0
+
+    def refcache_destroy(self, h):
+        pass
+
+
+@pytest.mark.parametrize("use", [contextlib.nullcontext, torch.no_grad, torch.inference_mode])
+@pytest.mark.parametrize("first", [contextlib.nullcontext, torch.no_grad, torch.inference_mode])
+def test_slot_views_can_be_written_whatever_mode_they_were_first_asked_for_in(monkeypatch, first, use):
+    c = rcb.RefCache.__new__(rcb.RefCache)
+    c.seg, c.num_layers, c.h = rcb.Segments(2, 64, [0, 1], [0, 5], [0]), 3, rcb.ctypes.c_void_p(1)
+    c.mem = torch.zeros(256 + 3 * 2 * 1280, dtype=torch.uint8)
+    monkeypatch.setattr(rcb, "load", lambda: _KvLibrary(c.mem.data_ptr()))
+    try:
+        with first():
+            c.kv(1)
+        x = torch.arange(5 * 2 * 64).view(5, 2, 64).to(torch.bfloat16)
+        with use():
+            for layer in (2, 0, 1, 2):
+                for i, slot in enumerate(c.kv(layer)):
+                    assert slot.shape == (5, 2, 64) and slot.data_ptr() == c.mem.data_ptr() + 256 + 1280 * (2 * layer + i)
+                    slot.copy_((x + layer + i).requires_grad_())
+                    assert torch.equal(c.kv(layer)[i], x + layer + i)
+        for bad in (-1, 3):
+            with pytest.raises(rcb.RefCacheError):
+                c.kv(bad)
+    finally:
+        c.h = None  # closed (and nothing for the library to free)
+    with pytest.raises(rcb.RefCacheError):
+        c.kv(0)
