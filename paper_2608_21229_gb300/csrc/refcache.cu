@@ -719,7 +719,8 @@ int cache_plan(int num_layers, int mode_flags, const refcache_segments_t* seg, r
       cp.push_back(c);
     }
   }
-  if (n_pieces > (1ll << 31) - 1) return fail(REFCACHE_ERR_INVALID_ARG, "cache rows too large");
+  if (h && n_pieces > (1ll << 31) - 1)  // (of 2 KB, twice a layer; refcache_bytes still answers)
+    return fail(REFCACHE_ERR_OOM, "a layer of more than 8 TB");
   order_tasks(bt);
   order_tasks(st);
   order_tasks(bs);

@@ -125,3 +125,12 @@ def test_workloads_of_the_split_tests_are_split_as_they_say(run_child, dim):
     # both forms of the merge: 16 blocks a job (8 at head dim 64), two of which fit on each of 152 SMs
     jobs = [len(o["jobs"]) * 8 * dim // 64 for o in out]
     assert min(jobs) <= 304 < max(jobs)
+
+
+def test_a_cache_too_large_to_build_can_still_be_planned(run_child):
+    """refcache_bytes is arithmetic: it answers for any rows that fit 32 bits."""
+    out = run_child("""
+seg = segments(8192, 128, [(0, 0, 1, 2147483000)])
+print(json.dumps([L.refcache_bytes(1, 0, ctypes.byref(seg.c)), L.refcache_bytes(2, 0, ctypes.byref(seg.c))]))""")
+    layer = 2 * 2147483000 * 8192 * 128 * 2
+    assert out[1] - out[0] == layer and 0 < out[0] - layer < 1 << 31
