@@ -1028,6 +1028,8 @@ int refcache_build(refcache_t* h, int layer, const void* q_static, const void* k
   if ((rc = enter_device(h, &info)) != 0) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   CacheWrite w;
+  if (h->n_qtiles > 65535)  // grid.y; it would be launched behind the prefill, and a refused call launches nothing
+    return fail(REFCACHE_ERR_CUDA, "quantize_cache_kernel launch: %d tiles of 128 cached rows, at most 65535", h->n_qtiles);
   if (h->n_qtiles > 0) {
     void *k8 = nullptr, *vt8 = nullptr, *sc = nullptr;
     refcache_fp8_ptr(h, layer, &k8, &vt8, &sc, nullptr);

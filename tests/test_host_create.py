@@ -134,3 +134,15 @@ seg = segments(8192, 128, [(0, 0, 1, 2147483000)])
 print(json.dumps([L.refcache_bytes(1, 0, ctypes.byref(seg.c)), L.refcache_bytes(2, 0, ctypes.byref(seg.c))]))""")
     layer = 2 * 2147483000 * 8192 * 128 * 2
     assert out[1] - out[0] == layer and 0 < out[0] - layer < 1 << 31
+
+
+def test_a_refused_build_launches_nothing(run_child):
+    """An E4M3 cache of more 128-row tiles than its cache write's grid takes (65535): the build says so before
+    it has launched the prefill."""
+    out = run_child("""
+seg, h = segments(1, 128, [(0, 0, 1, 1)] * 65536), ctypes.c_void_p()
+assert L.refcache_create(ctypes.byref(h), 1, 0x100, ctypes.byref(seg.c), None, 0) == 0
+t = ctypes.c_void_p(1 << 20)
+code = L.refcache_build(h, 0, t, t, t, t, None, 0.1, None)
+print(json.dumps([code, rc.last_error(), cudart.host_cudart_launches(), L.refcache_layer_built(h, 0)]))""")
+    assert out[0] == -4 and out[2] == 0 and out[3] == 0 and "quantize_cache_kernel" in out[1], out
