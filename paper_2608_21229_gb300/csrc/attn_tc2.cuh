@@ -436,13 +436,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
   // A cache's lists were written when it was created: the pair's first item need
   // not wait for the kernel before this one (0.7 us of the 2.5 us from the end of
   // that wait to the first MMA).
-  bool first_keys = false;
   if (args.static_list && leader && warp == Cfg::kProducerWarp && lane == 0) {
     Task t;
     int head;
     fetch_item(cluster, t, head);
     publish(0, t, head, 0);
-    first_keys = t.a_len + t.b_len > 0;
   }
   // launched as a programmatic dependent of the previous kernel on the stream:
   // everything above overlaps its tail, nothing below reads memory before it
@@ -460,21 +458,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
     // and K_t+2, which may belong to the next item, so that an item's first
     // loads are in flight before the item before it ends.
     if (lane == 0) {
-      // K and V tiles loaded (Q tiles: qi, scales: si), from which the loads of
+      // Q, K and V tiles loaded (scales: si), from which the loads of
       // every slot follow, and the kind of the last load of each slot; the leader
       // arms every phase for both CTAs' bytes right before it issues its own half.
       // (Kept per slot, in arrays, they lay in local memory, at hundreds of cycles
       // an access: the E4M3 kernel's producer took 11000 cycles from its last load
       // to its end and held up the pair's.  Step with 256 live and 256 cached rows,
       // 4 heads, E4M3: 21.4 us; now 9.7.  4608 and 20480, 24 heads: 911; now 892.)
-      int nk = 0, nv = 0;
+      int nq = 0, nk = 0, nv = 0;
       uint32_t last8 = 0;
       const bool skip = leader && args.dbg_skip_first_load != 0;
       int si = 0;  // cached tiles whose scales went into the ring
       // The leader's choice of the next item, in three steps, each of whose
       // result is first used by the following one: its index, its Task, its
       // publication.
-      int n_pub = args.static_list ? 1 : 0, pub_step = 0, pub_item = 0, pub_head = 0, pub_q = first_keys ? 1 : 0;
+      int n_pub = args.static_list ? 1 : 0, pub_step = 0, pub_item = 0, pub_head = 0;
       bool pub_end = false;
       Task pub_task{};
       auto pub_advance = [&]() -> bool {
@@ -493,9 +491,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           if (k >= tc2::kItemSlots &&
               !wait_cl_acquire(bar(L::kItemEmpty + s), static_cast<uint32_t>(k / tc2::kItemSlots - 1) & 1u, ctl, 21))
             return false;
-          publish(k, pub_task, pub_head, pub_q & 1);
+          publish(k, pub_task, pub_head, k & 1);
           pub_end = pub_head < 0;
-          if (pub_task.a_len + pub_task.b_len > 0) ++pub_q;
           ++n_pub;
         }
         pub_step = pub_step == 2 ? 0 : pub_step + 1;
@@ -503,7 +500,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       };
       // The K side: item k_item - 1, of which K tiles [0, kj) are loaded.
       Task kt{};
-      int k_item = 0, kj = 0, k_na = 0, k_nkv = 0, qi = 0;
+      int k_item = 0, kj = 0, k_na = 0, k_nkv = 0;
       bool k_end = false;
       // The V side: item v_item - 1, tile vj of it is next; G its group of S_1.
       Task vt{};
@@ -512,16 +509,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
 #pragma unroll 1
       for (int t = -2;; ++t) {  // V_t (from t = 0 on), then K_t+2
         if (t >= 0) {
-          while (vj == v_nkv) {  // the next item (the K side has passed it, so it is in the ring)
-            G += v_nkv > 0 || v_item == 0 ? v_nkv + 1 : 0;
+          if (vj == v_nkv) {  // the next item (the K side has passed it, so it is in the ring)
+            G += v_nkv + 1;
             vt = ring_read(v_item);
             if (!leader) ring_done(v_item);
             ++v_item;
-            vj = v_nkv = 0;
             if (vt.head < 0) break;
             v_nkv = tc2::n_key_tiles<kBN>(vt, v_na);
+            vj = 0;
           }
-          if (vt.head < 0) break;
           // The slots of V_t and K_t+2 are free once the P.V of tile t - kStages
           // and the S of tile t + 2 - kStages are complete.  Both hold after the
           // group below, which lies at most four groups before the first that
@@ -548,31 +544,30 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         }
         // the K side's next item, once its tiles are loaded; the leader chooses
         // the item after it from its last tiles on, one step per tile
-        for (;;) {
-          const bool need = !k_end && kj == k_nkv;
-          bool more = leader && !pub_end && n_pub <= k_item && kj + 3 >= k_nkv;
-          while (more) {
-            if (!pub_advance()) goto producer_done;
-            more = need && n_pub <= k_item;
-          }
-          if (!need) break;
+        const bool need = !k_end && kj == k_nkv;
+        bool more = leader && !pub_end && n_pub <= k_item && kj + 3 >= k_nkv;
+        while (more) {
+          if (!pub_advance()) goto producer_done;
+          more = need && n_pub <= k_item;
+        }
+        if (need) {
           if (!ring_wait(k_item, 18)) goto producer_done;
-          kt = ring_read(k_item++);
+          kt = ring_read(k_item);
           k_end = kt.head < 0;
-          if (k_end) break;
-          k_nkv = tc2::n_key_tiles<kBN>(kt, k_na);
-          kj = 0;
-          if (k_nkv == 0) continue;
-          const int b = qi & 1;  // its query rows into Q buffer qi % 2
-          const uint32_t n = static_cast<uint32_t>(qi >> 1);
-          if (!wait_one(bar(L::kQEmpty + b), (n & 1u) ^ 1u, ctl, 1)) goto producer_done;
-          if (leader) mbar_arrive_expect_tx(bar(L::kQFull + b), 2 * kQBoxes * kBoxBytes);
-          const uint32_t qfull = lbar(L::kQFull + b);
-          for (int ch = 0; ch < kQBoxes; ++ch)
-            tma_load_2d_pair(base + L::kQ + b * kQTile + ch * kBoxBytes, &tm_q, qfull, kt.head * DG + ch * 64,
-                             kt.q_row0 + 128 * static_cast<int>(rank));
-          ++qi;
-          break;
+          if (!k_end) {
+            k_nkv = tc2::n_key_tiles<kBN>(kt, k_na);
+            kj = 0;
+            const int b = k_item & 1;  // its query rows into Q buffer k_item % 2
+            const uint32_t n = static_cast<uint32_t>(k_item >> 1);
+            ++k_item;
+            if (!wait_one(bar(L::kQEmpty + b), (n & 1u) ^ 1u, ctl, 1)) goto producer_done;
+            if (leader) mbar_arrive_expect_tx(bar(L::kQFull + b), 2 * kQBoxes * kBoxBytes);
+            const uint32_t qfull = lbar(L::kQFull + b);
+            for (int ch = 0; ch < kQBoxes; ++ch)
+              tma_load_2d_pair(base + L::kQ + b * kQTile + ch * kBoxBytes, &tm_q, qfull, kt.head * DG + ch * 64,
+                               kt.q_row0 + 128 * static_cast<int>(rank));
+            ++nq;
+          }
         }
         if (k_end) continue;
         const int slot = slot_of(t + 2);
@@ -614,7 +609,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       const uint32_t rec = mapa_shared(base + L::kLoadRec + rank * (L::kRecWords * 4u), 0);
       st_cluster_u32(rec + 4u * L::kRecK, static_cast<uint32_t>(nk));
       st_cluster_u32(rec + 4u * L::kRecV, static_cast<uint32_t>(nv));
-      st_cluster_u32(rec + 4u * L::kRecQ, static_cast<uint32_t>(qi));
+      st_cluster_u32(rec + 4u * L::kRecQ, static_cast<uint32_t>(nq));
       st_cluster_u32(rec + 4u * L::kRecLast8, last8);
       st_cluster_u32(rec + 4u * L::kRecSkipped, skip && nk > 0 ? 1u : 0u);
       // this cluster takes no more items
@@ -785,22 +780,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       volatile int* gate_item = reinterpret_cast<volatile int*>(base_ptr + L::kGateItem);
       auto wait_k = [&](int t) -> bool { return wait_cl_warp(bar(L::kKFull + slot_of(t)), slot_parity(t), ctl, 4); };
       // the steps of the MMA warp (see there)
-      int nkv = -1, na = 0, nkv_next = 0, na_next = 0, k = 0, q8i = 0;
+      int nkv = -1, na = 0, nkv_next = 0, na_next = 0, q8i = 0;
 #pragma unroll 1
       for (int t0 = 0, qi = -1, j = -2;;) {
         const int t = t0 + j;
         bool ok = true;
         bool k_wait = j + 2 < nkv;
-        if (j + 2 == max(nkv, 0)) {  // name the next item with keys
-          for (;;) {
-            ok = ok && __all_sync(0xffffffffu, ring_wait(k, 19));
-            if (!ok) break;
+        if (j + 2 == max(nkv, 0)) {  // name the next item
+          const int k = qi + 1;
+          ok = ok && __all_sync(0xffffffffu, ring_wait(k, 19));
+          if (ok) {
             const Task tk = ring_read(k);
             __syncwarp();
             if (lane == 0) ring_done(k);
-            ++k;
             nkv_next = tk.head < 0 ? 0 : tc2::n_key_tiles<kBN>(tk, na_next);
-            if (tk.head < 0 || nkv_next > 0) break;
           }
           if (lane == 0) {
             volatile int* named = gate_item + 4 * ((qi + 1) & 1);
@@ -868,17 +861,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       const int nkv = tc2::n_key_tiles<kBN>(tk, na);
       const bool row_ok = prow < (tk.q_rows & 0xFFFF);
       const int64_t grow = static_cast<int64_t>(tk.q_row0) + prow;
-      if (nkv == 0) {
-        if (row_ok) {
-          __nv_bfloat16* orow = args.out + grow * args.row_stride + static_cast<int64_t>(head) * DG;
-          uint4 z = make_uint4(0, 0, 0, 0);
-          for (int c = 0; c < DG / 8; ++c) reinterpret_cast<uint4*>(orow)[c] = z;
-          if (args.lse) args.lse[grow * args.num_heads + head] = -INFINITY;
-        }
-        __syncwarp();
-        if (lane == 0) ring_done(k);
-        continue;
-      }
       float m_run = 0.f, l_run = 0.f;
       // E4M3 cache: this row's query scale (folded into sl2) and the weight scale s_ref
       float c_row = sl2, s_ref = 1.f, l2_ref = 0.f;

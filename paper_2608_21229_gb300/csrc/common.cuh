@@ -10,6 +10,7 @@
 //   full (rows [LT; X_t; R])       A = the request's whole sequence
 // so the mask is never materialised: a key is visible exactly when it lies in
 // A or B, and keys past the end of a range are cut off inside the last tile.
+// Every row sees a key at least (itself), so no task is without.
 // A launch enumerates items = tasks x heads, item i -> head i / n_tasks, task
 // i % n_tasks; or, when AttnArgs::per_item is set, an explicit list with one
 // task per item that names its head.  Such a list can also hold *parts* of an

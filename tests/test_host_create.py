@@ -39,11 +39,14 @@ def create(heads, dim, reqs, flags=0, fail_at=-1):
     out = dict(code=code, calls=cudart.host_cudart_calls().decode(), live=cudart.host_cudart_live())
     if code == 0:
         out["step_launches"] = L.refcache_call_launches(h, 1)
-        # after the memset: the build's items, the step's, its merge jobs (if any), the in-slot build's tasks (if any)
+        # after the memset: the build's items, the step's, its merge jobs, the in-slot build's tasks, each if there are any
+        lists = []
+        for i in range(out["calls"].index("s") + 1, out["calls"].rindex("m") + 1):
+            words = (ctypes.c_int32 * (cudart.host_cudart_copy_bytes(i) // 4)).from_address(cudart.host_cudart_copy_dst(i))
+            lists.append([list(words[k:k + 8]) for k in range(0, len(words), 8)])
         if out["step_launches"] == 2:
-            i = out["calls"].index("s") + 3
-            jobs = (ctypes.c_int32 * (cudart.host_cudart_copy_bytes(i) // 4)).from_address(cudart.host_cudart_copy_dst(i))
-            out["jobs"] = [list(jobs[k:k + 5]) for k in range(0, len(jobs), 8)]  # q_row0, q_rows, head, part0, nparts
+            out["jobs"] = lists.pop(2)  # q_row0, q_rows, head, part0, nparts
+        out["tasks"] = sum(lists, [])  # q_row0, q_rows, a_row0, a_len, b_row0, b_len, head, part
         L.refcache_destroy(h)
     out["live_after"] = cudart.host_cudart_live()
     return out
@@ -146,3 +149,18 @@ t = ctypes.c_void_p(1 << 20)
 code = L.refcache_build(h, 0, t, t, t, t, None, 0.1, None)
 print(json.dumps([code, rc.last_error(), cudart.host_cudart_launches(), L.refcache_layer_built(h, 0)]))""")
     assert out[0] == -4 and out[2] == 0 and out[3] == 0 and "quantize_cache_kernel" in out[1], out
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2])
+def test_every_item_has_rows_and_keys(run_child, mode):
+    """The pair kernel walks an item's key tiles without asking whether it has any: requests with empty blocks, in
+    every mask mode and cache type, and with parts, make no item without."""
+    lens = [0, 1, 5, 200, 1100]
+    reqs = [(a if mode != 2 else 0, b, c, d) for a in (0, 3) for b in lens[:3] for c in lens for d in lens]
+    big = [(0, 7, 230, 8300), (0, 0, 0, 0), (0 if mode == 2 else 4, 0, 1, 0)]
+    out = run_child(f"""
+outs = [create(2, 128, r, {mode} | f) for r in ({reqs}, {big}) for f in (0, 0x100)]
+print(json.dumps([dict(code=o["code"], jobs=len(o.get("jobs", [])), tasks=o["tasks"]) for o in outs]))""")
+    assert all(o["code"] == 0 and o["tasks"] for o in out) and any(o["jobs"] for o in out)
+    for o in out:
+        assert all(1 <= t[1] <= 256 and min(t[3], t[5]) >= 0 and t[3] + t[5] >= 1 for t in o["tasks"])
