@@ -305,8 +305,8 @@ def run_ours(args, ws, rank, local):
 
     def roof(flops, secs):
         """One kernel's (or sequence's) roofline figures against the measured
-        burst peak (the kernels here run near the maximum SM clock; the
-        sustained figure was measured at a lower, power-capped clock)."""
+        burst peak (a short loop; the sustained figure was measured under the
+        power cap, at a lower clock than these kernels run at)."""
         a = flops / secs / 1e12
         return {"achieved": a, "peak": peak, "unit": "TFLOP/s", "frac": a / peak}
     traffic = recorded_traffic(w.name, args.kernel) if args.cache == "bf16" else None
@@ -359,12 +359,12 @@ def run_ours(args, ws, rank, local):
                        + (")" if D == 128 else ", head dim 64)")) + " in step_attention",
             "bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
             "frac": achieved / peak,
-            "peak_kind": (f"bf16 dense, {pk['source']} burst (the timed region runs near the maximum SM clock)"
+            "peak_kind": (f"bf16 dense, {pk['source']} burst (a short loop; the timed region's SM clock is in clocks)"
                           if args.cache == "bf16" else
                           f"E4M3 dense = 2 x bf16 {pk['source']} burst (nominal ratio)"),
             "frac_of_sustained": achieved / (peak_mult * pk["bf16_sustained"]),
-            "sustained_note": "the sustained peak was measured at a power-capped median SM clock of about "
-                              "1.4 GHz; this kernel's timed region runs near 2 GHz, so it is context only",
+            "sustained_note": "the sustained peak was measured in a loop of seconds under the power cap, at a lower "
+                              "SM clock than the timed region's (in clocks), so it is context only",
             "nominal_at_clock": nominal_at_clock(achieved, clocks.get("sm_mhz"), sms, peak_mult),
             "exp_floor": exp_floor(acc.step_units(w.requests) * H, t_step, clocks.get("sm_mhz"), sms, ex2_rate),
             "traffic": traffic,

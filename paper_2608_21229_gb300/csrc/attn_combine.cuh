@@ -33,13 +33,13 @@ constexpr int kCombineRows = 32;
 // that fit on an SM (57 registers against 92): a block takes all columns, part after
 // part.  us a call, back to back, 256 rows of 128 columns, ahead / part after part:
 //   jobs     2 parts       4 parts        8 parts
-//      4   2.0 /  2.7    2.1 /  3.4     2.4 /  4.4
-//     12   2.3 /  2.7    2.4 /  3.5     2.8 /  4.5
-//     18   2.4 /  2.8    2.5 /  3.6     3.0 /  4.6
-//     24   3.7 /  2.9    3.9 /  3.7     4.8 /  4.9
-//     76   7.5 /  3.9    8.2 /  5.0    10.5 /  7.1
-// (Step with 256 live and 8192 cached rows, 4 heads, 8 parts: 17.6 us part after
-// part, now 13.8; on an E4M3 cache 20.1, now 17.0.)
+//      4   2.0 /  2.7    2.1 /  3.5     2.4 /  4.6
+//     12   2.4 /  2.8    2.5 /  3.6     2.9 /  4.7
+//     18   2.4 /  2.9    2.6 /  3.7     3.1 /  4.8
+//     24   3.5 /  3.0    4.0 /  3.8     4.8 /  5.1
+//     76   7.2 /  4.0    7.7 /  5.2    10.6 /  7.4
+// (A step with 256 live and 8192 cached rows, 4 heads, 8 parts: 17.6 us part after
+// part, 13.8 ahead.)
 // The line (launch_combine) lies where the blocks of the first form fill two per SM.
 template <int D, int kQ, bool kAhead>
 __global__ void __launch_bounds__(256) combine_parts_kernel(const CombineJob* __restrict__ jobs,

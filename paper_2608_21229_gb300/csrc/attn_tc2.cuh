@@ -60,9 +60,8 @@
 // the item, passing it to the other CTA and reading its Task from global memory
 // in every role one after the other took about 5000 cycles per item, and the
 // epilogue's uncoalesced stores 2000.  MMA-thread waits around an item's start
-// went from 5100 to 2700 cycles; step with 1280 live and 2048 cached rows
-// (items of 9 tiles), 24 heads: 62.7 -> 60.7 us (its last round was still split then;
-// now 43 us).
+// went from 5100 to 2700 cycles, 3 % of a step with 1280 live and 2048 cached
+// rows and 24 heads (items of 18 tiles).
 //
 // Synchronisation is built so that the MMA thread waits on nothing itself: all
 // mbarrier waits are done by the gate warp: per group, the gate warp waits for
@@ -100,10 +99,8 @@
 // period: 1880 cycles per tile at 4608 live and 20480 cached rows, 24 heads, of
 // which the MMA thread waited 480 for P.  With the first 96 keys handed over
 // early, their handshake and their P.V MMAs leave the loop.  Cycles per tile by
-// the size of the first piece: 32 keys 1743, 64 keys 1700, 96 keys 1697, 128
-// keys 1711 (with the MMAs under elect.sync 1678, 1635 and 1641 for 64, 96 and
-// 128 keys; 32 keys measured best while the softmax warps still took 300 cycles
-// more per tile than now).
+// the size of the first piece: 64 keys 1678, 96 keys 1635, 128 keys 1641 (32 keys,
+// with the MMAs under lane == 0, 46 more than 96).
 //
 // The softmax warps are as long in a tile (about 1550 cycles: loads and maximum
 // 215, exponentials and P 1180 of which the exponential unit needs 800, the rest
@@ -279,9 +276,9 @@ __device__ __forceinline__ void work_done(int* work, int n_clusters) {
 // rows with the 64-byte swizzle, P V with N = 64, O in 64 columns of tensor
 // memory.  (Padded to 128 columns, with zeros for the second CTA's half, P V did
 // twice the work.  The softmax warps bound this head dim, but the MMAs lie on the
-// way from P to the next S: in-place build of three requests with 48 heads, 1614
-// to 6271 rows, 574 -> 544 us; step of 320 live and 256 cached rows, 4 heads,
-// 8.89 -> 8.72 us.)
+// way from P to the next S: unpadded, an in-place build of three requests with 48
+// heads, 1614 to 6271 rows, takes 5 % less, a step of 320 live and 256 cached rows
+// with 4 heads 2 %.)
 template <bool kF8, int kBN, int kDG>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::kThreads, 1)
     attn_tc2_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_ka,
@@ -463,8 +460,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
       // arms every phase for both CTAs' bytes right before it issues its own half.
       // (Kept per slot, in arrays, they lay in local memory, at hundreds of cycles
       // an access: the E4M3 kernel's producer took 11000 cycles from its last load
-      // to its end and held up the pair's.  Step with 256 live and 256 cached rows,
-      // 4 heads, E4M3: 21.4 us; now 9.7.  4608 and 20480, 24 heads: 911; now 892.)
+      // to its end and held up the pair's: 21.4 us a step with 256 live and 256
+      // cached rows and 4 heads, 9.7 without; 2 % with 4608 and 20480, 24 heads.)
       int nq = 0, nk = 0, nv = 0;
       uint32_t last8 = 0;
       const bool skip = leader && args.dbg_skip_first_load != 0;
@@ -942,8 +939,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
         // loads deliver the maximum of each 32 columns (tcgen05.ld.red).  The
         // maximum sits on the latency loop that bounds the kernel (S ready ->
         // softmax -> P -> next S): with 96 max instructions per 192-key tile it
-        // took about 190 of 2142 cycles.  Step at 4608 live and 20480 cached
-        // rows, 24 heads: 898 -> 838 us, same bits.
+        // took about 190 of 2142 cycles, and the step at 4608 live and 20480 cached
+        // rows, 24 heads, 7 % longer (same bits).
         float s[kBN];
         float m_raw;
         {
@@ -993,8 +990,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           m_run = m_new;
           l_run *= alpha;
           const uint32_t t_o = tmem + lane_off + kColO;
-          // (rolled in the E4M3 kernel: 919 -> 896 us at 4608 live and 20480 cached
-          // rows, 24 heads; the bf16 kernel is 0.5-1.5 % faster unrolled)
+          // (rolled in the E4M3 kernel, whose tile loop holds the code of both kinds
+          // of tile; rolled, by two or unrolled, both kernels take the same time within
+          // 0.7 %)
           constexpr int kUnroll = kF8 ? 1 : DG / 16;
 #pragma unroll kUnroll
           for (int cc = 0; cc < DG / 16; ++cc) {
@@ -1032,8 +1030,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc2::Cfg<kF8, kBN>::
           for (int i = 0; i < 4; ++i) lacc[i] = make_f32x2(0.f, 0.f);
           if (t8) {
             // the next tile's scales are looked for and read on the way (waited for
-            // and read at its start they took 345 cycles of a tile's 1490: 967 us a
-            // step instead of 920)
+            // and read at its start they took 345 cycles of a tile's 1490, 5 % of a
+            // step)
             const int sl = si % tc2::kScaleSlots;
             bool found = false;
 #pragma unroll

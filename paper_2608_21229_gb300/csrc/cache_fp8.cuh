@@ -53,13 +53,13 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 // rows [8 g, 8 g + 8) of column d is word g ^ ((d / 8) % 16) of the column's 128
 // bytes, which spreads both the stores (16 columns 8 apart) and the reads (a
 // column's 128 bytes) over all banks.  (With a lane per four rows each load and K
-// store touched 32 rows' sectors: build of a 1024^2 request with two references
-// 541 us, 42 of them here; now 525.)
+// store touched 32 rows' sectors, and the build of a 1024^2 request with two
+// references, 42 us of it here, took 3 % longer.)
 //
 // Like copy_rows_kernel it reads only the static inputs and goes behind the
 // prefill as its programmatic dependent: its CTAs fill in as the prefill's leave.
-// (Before the prefill: build of nine heads, two requests of 740 and 5694 cached
-// rows, 112 us; behind it 107.)
+// (Before the prefill a build of nine heads, two requests of 740 and 5694 cached
+// rows, took 112 us, behind it 107.)
 struct QuantArgs {
   const QuantTile* tiles;
   int32_t n_tiles, num_heads;

@@ -476,12 +476,13 @@ double list_end(const std::map<double, int64_t, std::greater<double>>& costs, in
 // of the persistent grid, the items of that round may be split by key tiles into
 // s parts each, which run after the whole items; their results are merged by
 // combine jobs.  Whether, and into how many, by the end of the list under these
-// costs, in key-tile times (0.8 us; measured on the kernel's timeline): an item's
-// start and epilogue 2 (E4M3: 6), a part's larger epilogue 1, and the combine
-// kernel 6 (its hand-overs with the attention kernels around it) plus 0.03 per
-// part.  (Splitting whenever the last round was not full cost the step with 1280
-// live and 2048 cached rows, 24 heads, 10 us in the combine and the parts to save
-// 6.)
+// costs, in key-tile times (0.8 us for the 192-key kernel at head dim 128, whose
+// timeline they were read from; the others use them as they are): an item's
+// start and epilogue 2 (E4M3: 6; 3 and 10 give the same times), a part's larger
+// epilogue 1, and the combine kernel 6 (its hand-overs with the attention kernels
+// around it) plus 0.03 per part.  (Splitting whenever the last round was not full
+// cost the step with 1280 live and 2048 cached rows, 24 heads, 10 us in the combine
+// and the parts to save 6.)
 void plan_items(const std::vector<Task>& tasks, int H, int clusters, int tile, bool f8, std::vector<Task>* items,
                 std::vector<CombineJob>* jobs, int* n_parts) {
   items->clear();
@@ -1141,8 +1142,8 @@ int full_attention(int batch, int num_heads, int head_dim, const int32_t* cu_seq
   const int tr = task_rows(head_dim);
   // Up to kMaxSpans requests go as a kernel parameter, longest first, so that no
   // list is copied on the stream: the copy and the full stop around it, where
-  // otherwise one call's prologue overlaps the tail of the one before, cost 8 us a
-  // call (5 heads, 1964 rows: 22.3 us; now 16.4).  (The mma.sync kernel reads a list.)
+  // otherwise one call's prologue overlaps the tail of the one before, cost 6 us a
+  // call (5 heads, 1964 rows: 22.3 us with, 16.4 without).  (The mma.sync kernel reads a list.)
   rc::Spans spans{};
   int64_t n_span_tasks = 0;
   if (g_kernel.load() != REFCACHE_KERNEL_MMA_SYNC && batch <= rc::kMaxSpans) {

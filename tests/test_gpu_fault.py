@@ -46,9 +46,9 @@ def test_wait_timeout_is_reported_and_context_survives():
 @pytest.mark.parametrize("cache_dtype", ["bf16", "fp8"])
 def test_pair_kernel_wait_timeout_is_reported_and_context_survives(cache_dtype):
     """The same on the head-dim-128 CTA-pair kernel (its gate, MMA, producer and
-    softmax warps in both CTAs, and for the E4M3 cache the query-tile, scale
-    ring and row-sum waits): the leader skips its first stage, every wait of
-    the pair runs out or sees the abort, and the next call is correct."""
+    softmax warps in both CTAs, and for the E4M3 cache the query-tile and scale
+    ring waits): the leader skips its first K tile, every wait of the pair runs
+    out or sees the abort, and the next call is correct."""
     rcb.load()
     rcb.set_kernel("tcgen05")
     w = workloads.CFG_SMALL
